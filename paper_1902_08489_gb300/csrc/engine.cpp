@@ -368,24 +368,12 @@ struct GemmBatch {
   std::vector<GemmSeg> segs;
   std::vector<SegOps> segops;
   double flops = 0.0, bytes = 0.0;
-  // a segmented task of an FP64 batch, expanded into one plain task per
-  // segment once its terms are known (the FP64 kernel has no segments)
-  struct PendSeg {
-    bool live = false;
-    GemmSeg s;
-    int other, tc, opA, ta, opB, tb;
-    bool beta;
-    cplx alpha;
-    struct T { const void* shared; int ld; SegOps so; int K; cplx scale; const double2* sp; };
-    std::vector<T> terms;
-  } pend;
   explicit GemmBatch(Context& ctx, bool force_fp64 = false)
       : c(ctx), fp64(force_fp64 || ctx.precision == TDMPS_FP64) {}
   // A task whose rows (dim 0) or columns (dim 1) are n output blocks of the
   // given sizes (GemmSeg); `other` is the extent of the other dimension.
   void task_seg(int dim, int n, void* const* Cs, const int* ldcs, const int* sizes, int other,
                 int tc, int opA, int ta, int opB, int tb, bool beta, cplx alpha) {
-    flush();
     if (n < 1 || n > 4) throw Error(TDMPS_ERR_INVALID_ARG, "a GEMM task holds 1 to 4 segments");
     GemmSeg s{};
     s.dim = dim;
@@ -396,14 +384,6 @@ struct GemmBatch {
       s.ldc[i] = ldcs[i];
     }
     for (int i = n; i < 4; ++i) s.off[i + 1] = s.off[i];
-    if (fp64) {
-      pend.live = true;
-      pend.s = s;
-      pend.other = other; pend.tc = tc; pend.opA = opA; pend.ta = ta; pend.opB = opB; pend.tb = tb;
-      pend.beta = beta; pend.alpha = alpha;
-      pend.terms.clear();
-      return;
-    }
     const int total = s.off[n];
     task(Cs[0], tc, dim == 0 ? total : other, dim == 0 ? other : total, ldcs[0], opA, ta, opB, tb,
          beta, alpha);
@@ -417,17 +397,13 @@ struct GemmBatch {
     if (K <= 0) return;
     SegOps so{};
     const void* any = nullptr;
-    const GemmSeg& s = pend.live ? pend.s : segs[tasks.back().seg1 - 1];
+    const GemmSeg& s = segs[tasks.back().seg1 - 1];
     for (int i = 0; i < s.n; ++i) {
       so.p[i] = segp[i];
       so.ld[i] = segld[i];
       if (segp[i] && !any) any = segp[i];
     }
     if (!any) return;
-    if (pend.live) {
-      pend.terms.push_back({shared, ld_shared, so, K, scale, scale_ptr});
-      return;
-    }
     GemmTask& t = tasks.back();
     GemmTerm g{};
     if (s.dim == 0) { g.A = any; g.B = shared; g.ldb = ld_shared; }
@@ -445,27 +421,10 @@ struct GemmBatch {
     for (int i = 0; i < s.n; ++i)
       if (segp[i]) live += s.off[i + 1] - s.off[i];
     flops += 8.0 * live * other * K;
-    bytes += 8.0 * (live * K + (double)other * K);
-  }
-  void flush() {
-    if (!pend.live) return;
-    pend.live = false;
-    const GemmSeg& s = pend.s;
-    for (int i = 0; i < s.n; ++i) {
-      const int sz = s.off[i + 1] - s.off[i];
-      if (sz <= 0) continue;
-      task(s.C[i], pend.tc, s.dim == 0 ? sz : pend.other, s.dim == 0 ? pend.other : sz, s.ldc[i],
-           pend.opA, pend.ta, pend.opB, pend.tb, pend.beta, pend.alpha);
-      for (const auto& tm : pend.terms) {
-        if (!tm.so.p[i]) continue;
-        if (s.dim == 0) term(tm.so.p[i], tm.so.ld[i], tm.shared, tm.ld, tm.K, tm.scale, tm.sp);
-        else term(tm.shared, tm.ld, tm.so.p[i], tm.so.ld[i], tm.K, tm.scale, tm.sp);
-      }
-    }
+    bytes += (t.ta ? 8.0 : 16.0) * (live * K + (double)other * K);
   }
   void task(void* C, int tc, int M, int N, int ldc, int opA, int ta, int opB, int tb, bool beta,
             cplx alpha, const double2* aptr = nullptr, const double2* adiv = nullptr) {
-    flush();
     if (fp64 && (ta || tb || tc)) throw Error(TDMPS_ERR_INVALID_ARG, "FP64 GEMM on float data");
     if (!fp64 && (!ta || !tb))
       throw Error(TDMPS_ERR_INVALID_ARG, "tensor-core GEMM operands must be complex float");
@@ -500,11 +459,12 @@ struct GemmBatch {
       default: return OP_C;
     }
   }
-  // FP64 tiles skip whole warps of rows past the block edge, so a task whose
-  // N is the short side runs transposed (rows <- the short side).
+  // The FP64 kernel pads rows to 16 and columns to 4, so a task runs
+  // transposed when that wastes less.
   void orient_fp64() {
+    auto up = [](long long x, int g) { return (x + g - 1) / g * g; };
     for (auto& t : tasks) {
-      if (t.M <= 0 || t.N <= 0 || t.N >= t.M || t.N >= 32) continue;
+      if (t.seg1 || t.M <= 0 || t.N <= 0 || up(t.N, 16) * up(t.M, 4) >= up(t.M, 16) * up(t.N, 4)) continue;
       for (int e = t.term_begin; e < t.term_end; ++e) {
         std::swap(terms[e].A, terms[e].B);
         std::swap(terms[e].lda, terms[e].ldb);
@@ -515,6 +475,97 @@ struct GemmBatch {
       std::swap(t.ta, t.tb);
       std::swap(t.M, t.N);
       t.ct = 1;
+    }
+  }
+  // A launch whose tiles (32 x 32, segments apart) are all of at most
+  // SMALL_MACS complex multiply-adds, and few enough for one wave of that
+  // size, runs on the FP64 pipe (0.43 of them per clock and SM: 9 us; the
+  // sliced kernel takes about as long for any tile).
+  static constexpr long long SMALL_MACS = 8192;
+  bool small_fp64() const {
+    long long total = 0;
+    for (const auto& t : tasks) {
+      long long k = 0;
+      for (int e = t.term_begin; e < t.term_end; ++e) k += terms[e].K;
+      int m = t.M, n = t.N;
+      if (t.seg1) {   // the largest segment
+        const GemmSeg& s = segs[t.seg1 - 1];
+        int w = 0;
+        for (int i = 0; i < s.n; ++i) w = std::max(w, s.off[i + 1] - s.off[i]);
+        (s.dim == 0 ? m : n) = w;
+      }
+      if (std::min(m, 32) * std::min(n, 32) * k > SMALL_MACS) return false;
+      total += (long long)t.M * t.N * k;
+    }
+    return total <= SMALL_MACS * std::max(1, c.n_sm);
+  }
+  // Segmented tasks as one plain task per segment (more, smaller tiles for
+  // the FP64 pipe), each with its short side as rows: warps of rows past the
+  // block edge do no arithmetic.
+  void expand_small() {
+    std::vector<GemmTask> tk;
+    std::vector<GemmTerm> tm;
+    tm.reserve(terms.size());
+    for (const auto& t0 : tasks) {
+      const GemmSeg* s = t0.seg1 ? &segs[t0.seg1 - 1] : nullptr;
+      for (int i = 0; i < (s ? s->n : 1); ++i) {
+        GemmTask t = t0;
+        t.seg1 = 0;
+        if (s) {
+          t.C = s->C[i];
+          t.ldc = s->ldc[i];
+          (s->dim == 0 ? t.M : t.N) = s->off[i + 1] - s->off[i];
+        }
+        if (t.M <= 0 || t.N <= 0) continue;
+        const bool flip = t.N < t.M && t.N < 32;
+        t.term_begin = (int)tm.size();
+        for (int e = t0.term_begin; e < t0.term_end; ++e) {
+          GemmTerm g = terms[e];
+          if (s) {
+            const SegOps& so = segops[g.pad];
+            if (!so.p[i]) continue;
+            if (s->dim == 0) { g.A = so.p[i]; g.lda = so.ld[i]; }
+            else { g.B = so.p[i]; g.ldb = so.ld[i]; }
+          }
+          if (flip) {
+            std::swap(g.A, g.B);
+            std::swap(g.lda, g.ldb);
+          }
+          tm.push_back(g);
+        }
+        t.term_end = (int)tm.size();
+        if (flip) {
+          t.opA = op_t(t0.opB);
+          t.opB = op_t(t0.opA);
+          std::swap(t.M, t.N);
+          t.ct = 1;
+        }
+        tk.push_back(t);
+      }
+    }
+    tasks.swap(tk);
+    terms.swap(tm);
+  }
+  // A coefficient that all terms of a task share multiplies its result
+  // instead of every element of A (four FP64 operations each).
+  void hoist_scale() {
+    for (auto& t : tasks) {
+      if (t.term_begin >= t.term_end) continue;
+      const GemmTerm f = terms[t.term_begin];
+      if (f.scale.x == 1.0 && f.scale.y == 0.0 && !f.scale_ptr) continue;
+      if (f.scale_ptr && t.alpha_ptr) continue;
+      bool same = true;
+      for (int e = t.term_begin; e < t.term_end && same; ++e)
+        same = terms[e].scale.x == f.scale.x && terms[e].scale.y == f.scale.y &&
+               terms[e].scale_ptr == f.scale_ptr;
+      if (!same) continue;
+      t.alpha = make_double2(t.alpha.x * f.scale.x - t.alpha.y * f.scale.y,
+                             t.alpha.x * f.scale.y + t.alpha.y * f.scale.x);
+      if (f.scale_ptr) t.alpha_ptr = f.scale_ptr;
+      for (int e = t.term_begin; e < t.term_end; ++e) {
+        terms[e].scale = make_double2(1.0, 0.0);
+        terms[e].scale_ptr = nullptr;
+      }
     }
   }
   // Tensor-core tiles are 128 rows (the MMA M) by up to 64 complex columns
@@ -539,10 +590,19 @@ struct GemmBatch {
     }
   }
   void run() {
-    flush();
-    const int bm = fp64 ? 32 : tc_tile_m();
-    const int bn = fp64 ? 32 : tc_tile_n();
-    if (fp64) orient_fp64(); else orient_tc();
+    bool small = false;
+    if (fp64) {
+      hoist_scale();
+      small = small_fp64();
+      if (small) expand_small(); else orient_fp64();
+    } else {
+      orient_tc();
+    }
+    const int bm = tc_tile_m(), bn = tc_tile_n();
+    auto tiles_m = [&](int M) { return fp64 ? f64_tiles_m(M, small) : (M + bm - 1) / bm; };
+    auto tiles_n = [&](const GemmTask& t) {
+      return fp64 ? f64_tiles_n(t.N, small, t.walk) : (t.N + bn - 1) / bn;
+    };
     std::vector<int> tile_task;
     std::vector<GemmTask> tk;
     std::vector<int> split_ids;
@@ -555,24 +615,26 @@ struct GemmBatch {
     // and the tensor pipe are per-SM resources; a launch with fewer units
     // than SMs leaves the rest idle), with at least `min_chunks` K chunks
     // per unit to amortise the partial-slice store and its reduction.
-    const int kc = fp64 ? 8 : tc_stage_k();
+    const int kc = fp64 ? f64_stage_k() : tc_stage_k();
     const int per_sm = fp64 ? 4 : 3, min_chunks = fp64 ? 2 : 4;
     std::vector<long long> stages(tasks.size(), 0);
     long long total = 0;
     for (size_t i = 0; i < tasks.size(); ++i) {
-      const GemmTask& t = tasks[i];
+      GemmTask& t = tasks[i];
       if (t.M <= 0 || t.N <= 0) continue;
       for (int e = t.term_begin; e < t.term_end; ++e) stages[i] += (terms[e].K + kc - 1) / kc;
-      total += (long long)((t.M + bm - 1) / bm) * ((t.N + bn - 1) / bn) * std::max(1LL, stages[i]);
+      const int nt = t.term_end - t.term_begin;
+      t.walk = fp64 && !small ? f64_walk(t.N, nt, nt ? terms[t.term_begin].K : 0) : 1;
+      total += (long long)tiles_m(t.M) * tiles_n(t) * std::max(1LL, stages[i]);
     }
     const long long units = (long long)std::max(1, c.n_sm) * per_sm;
     const long long chunk = std::max<long long>(min_chunks, total / units);
     for (size_t i = 0; i < tasks.size(); ++i) {
       GemmTask& t = tasks[i];
       if (t.M <= 0 || t.N <= 0) continue;
-      t.tiles_m = (t.M + bm - 1) / bm;
-      int tn = (t.N + bn - 1) / bn;
-      t.splits = (int)std::min<long long>(64, std::max<long long>(1, stages[i] / chunk));
+      t.tiles_m = tiles_m(t.M);
+      const int tn = tiles_n(t);
+      t.splits = t.walk > 1 ? 1 : (int)std::min<long long>(64, std::max<long long>(1, stages[i] / chunk));
       t.part = nullptr;
       t.tile_base = (int)tile_task.size();
       int id = (int)tk.size();
@@ -667,7 +729,8 @@ struct GemmBatch {
     const int kind = fp64 ? TDMPS_KSTAT_GEMM_FP64 : TDMPS_KSTAT_GEMM;
     c.kbegin(kind, &ev);
     if (fp64)
-      launch_gemm(dt, (int)tk.size(), dm, dtt, (int)tile_task.size(), c.st);
+      launch_gemm(dt, dm, (const GemmSeg*)(base + o_segs), (const SegOps*)(base + o_segops), dtt,
+                  (int)tile_task.size(), small, c.st);
     else
       launch_gemm_tc(dt, dm, (const TcTile*)(base + o_tiles), (const GemmSeg*)(base + o_segs),
                      (const SegOps*)(base + o_segops), (int)tc_tiles.size(),

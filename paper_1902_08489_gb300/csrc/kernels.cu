@@ -1,5 +1,4 @@
-// FP64 device kernels of the tdmps library: grouped complex block GEMM, sparse
-// MPO-tensor application, block gather/scatter, one-sided Jacobi SVD, Gram-Schmidt
+// FP64 device kernels of the tdmps library: sparse MPO-tensor application, block gather/scatter, one-sided Jacobi SVD, Gram-Schmidt
 // QR, the truncation rule, and the small Krylov algebra.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
@@ -50,118 +49,6 @@ __device__ __forceinline__ double2 cdiv(double2 a, double2 b) {
 __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
-}
-
-// ------------------------------------------------------------------ grouped GEMM
-
-constexpr int GT = 32;    // output tile edge
-constexpr int GK = 8;     // K chunk
-
-__device__ __forceinline__ double2 load_op(const double2* P, int ld, int op, int r, int c,
-                                           int R, int C) {
-  // element (r, c) of op(P) where op(P) is R x C
-  if (r >= R || c >= C) return make_double2(0.0, 0.0);
-  switch (op) {
-    case OP_N: return P[(size_t)r * ld + c];
-    case OP_T: return P[(size_t)c * ld + r];
-    case OP_C: return cconj(P[(size_t)c * ld + r]);
-    default: return cconj(P[(size_t)r * ld + c]);
-  }
-}
-
-__global__ void __launch_bounds__(256) k_gemm(const GemmTask* __restrict__ tasks,
-                                              const GemmTerm* __restrict__ terms,
-                                              const int* __restrict__ tile_task) {
-  __shared__ double2 As[GK][GT + 1];
-  __shared__ double2 Bs[GK][GT + 1];
-  const int ti = tile_task[blockIdx.x];
-  const GemmTask t = tasks[ti];
-  const int local = blockIdx.x - t.tile_base;
-  const int split = local % t.splits;
-  const int rest = local / t.splits;
-  const int m0 = (rest % t.tiles_m) * GT;
-  const int n0 = (rest / t.tiles_m) * GT;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  // rows past the block edge do no arithmetic (a warp covers 4 rows, so a
-  // short block leaves whole warps idle instead of multiplying zeros)
-  const bool rows_live = m0 + 2 * ty < t.M;
-  double2 acc[2][2];
-  for (int i = 0; i < 2; ++i)
-    for (int j = 0; j < 2; ++j) acc[i][j] = make_double2(0.0, 0.0);
-  // this split's share of the task's K chunks (GK each, over all terms)
-  int S = 0;
-  for (int e = t.term_begin; e < t.term_end; ++e) S += (terms[e].K + GK - 1) / GK;
-  const int lo = (int)((long long)split * S / t.splits);
-  const int hi = (int)((long long)(split + 1) * S / t.splits);
-  int idx = 0;
-  for (int e = t.term_begin; e < t.term_end && idx < hi; ++e) {
-    const GemmTerm g = terms[e];
-    const int nk = (g.K + GK - 1) / GK;
-    if (idx + nk <= lo) { idx += nk; continue; }
-    double2 sc = g.scale;
-    if (g.scale_ptr) sc = cmul(sc, *g.scale_ptr);
-    const int c0 = lo > idx ? lo - idx : 0;
-    const int c1 = hi - idx < nk ? hi - idx : nk;
-    for (int ch = c0; ch < c1; ++ch) {
-      const int k0 = ch * GK;
-      {
-        int i = threadIdx.x >> 3, k = threadIdx.x & 7;      // A tile: 32 x 8
-        As[k][i] = cmul(sc, load_op((const double2*)g.A, g.lda, t.opA, m0 + i, k0 + k, t.M, g.K));
-        int kk = threadIdx.x >> 5, j = threadIdx.x & 31;    // B tile: 8 x 32
-        Bs[kk][j] = load_op((const double2*)g.B, g.ldb, t.opB, k0 + kk, n0 + j, g.K, t.N);
-      }
-      __syncthreads();
-      if (rows_live) {
-        if (k0 + GK <= g.K) {
-#pragma unroll
-          for (int k = 0; k < GK; ++k) {
-            double2 a0 = As[k][ty * 2], a1 = As[k][ty * 2 + 1];
-            double2 b0 = Bs[k][tx * 2], b1 = Bs[k][tx * 2 + 1];
-            acc[0][0] = cfma(a0, b0, acc[0][0]);
-            acc[0][1] = cfma(a0, b1, acc[0][1]);
-            acc[1][0] = cfma(a1, b0, acc[1][0]);
-            acc[1][1] = cfma(a1, b1, acc[1][1]);
-          }
-        } else {   // ragged last chunk: only the valid K
-          const int kl = g.K - k0;
-          for (int k = 0; k < kl; ++k) {
-            double2 a0 = As[k][ty * 2], a1 = As[k][ty * 2 + 1];
-            double2 b0 = Bs[k][tx * 2], b1 = Bs[k][tx * 2 + 1];
-            acc[0][0] = cfma(a0, b0, acc[0][0]);
-            acc[0][1] = cfma(a0, b1, acc[0][1]);
-            acc[1][0] = cfma(a1, b0, acc[1][0]);
-            acc[1][1] = cfma(a1, b1, acc[1][1]);
-          }
-        }
-      }
-      __syncthreads();
-    }
-    idx += nk;
-  }
-  double2 alpha = t.alpha;
-  if (t.alpha_ptr) alpha = cmul(alpha, *t.alpha_ptr);
-  if (t.alpha_div) alpha = cdiv(alpha, *t.alpha_div);
-  for (int i = 0; i < 2; ++i)
-    for (int j = 0; j < 2; ++j) {
-      int r = m0 + ty * 2 + i, c = n0 + tx * 2 + j;
-      if (r < t.M && c < t.N) {
-        double2* p = (double2*)t.C + (t.ct ? (size_t)c * t.ldc + r : (size_t)r * t.ldc + c);
-        double2 v = cmul(alpha, acc[i][j]);
-        if (t.splits > 1) {
-          ((double2*)t.part)[((size_t)split * t.M + r) * t.N + c] = v;
-        } else {
-          if (t.beta) v = cadd(v, *p);
-          *p = v;
-        }
-      }
-    }
-}
-
-void launch_gemm(const GemmTask* d_tasks, int ntasks, const GemmTerm* d_terms,
-                 const int* d_tile_task, int ntiles, cudaStream_t st) {
-  (void)ntasks;
-  if (ntiles <= 0) return;
-  k_gemm<<<ntiles, 256, 0, st>>>(d_tasks, d_terms, d_tile_task);
 }
 
 // ------------------------------------------------------------------ W stage

@@ -41,8 +41,9 @@ struct GemmTask {
   // double from the FP64 kernel) and launch_reduce_splits adds the slices in
   // split order into C, so results do not depend on timing
   void* part;
-  // tensor-core path: 1 + index of this task's GemmSeg (0: not segmented)
+  // 1 + index of this task's GemmSeg (0: not segmented)
   int seg1;
+  int walk;              // FP64 kernel: column tiles of one CTA
 };
 
 // A segmented task: the rows (dim 0) or the columns (dim 1) of C are the
@@ -107,8 +108,17 @@ struct FactTask {
   int m, n;
 };
 
-void launch_gemm(const GemmTask* d_tasks, int ntasks, const GemmTerm* d_terms,
-                 const int* d_tile_task, int ntiles, cudaStream_t st);
+// FP64 grouped GEMM (kernels_f64.cu): one CTA per split and tile; d_tile_task
+// names the task of every CTA, the CTAs of a task in (split, row, column)
+// order.  A CTA covers one row tile and t.walk column tiles.
+// small: the kernel on the FP64 pipe, for launches of little work (plain tasks).
+int f64_tiles_m(int M, bool small);              // row tiles of a task
+int f64_tiles_n(int N, bool small, int walk);    // CTAs along its columns
+int f64_walk(int N, int nterms, int K);   // column tiles per CTA: several when one K group is all
+int f64_stage_k();                  // complex K per step; split-K shares out whole steps
+void launch_gemm(const GemmTask* d_tasks, const GemmTerm* d_terms, const GemmSeg* d_segs,
+                 const SegOps* d_segops, const int* d_tile_task, int ntiles, bool small,
+                 cudaStream_t st);
 // et: element type of X and Y (0 double2 with the FP64 values, 1 float2 with
 // the FP32 copy of the values)
 // rows a of a W-stage block that one work item covers (work per block:

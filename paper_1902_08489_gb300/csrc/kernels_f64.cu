@@ -1,0 +1,570 @@
+// Grouped complex FP64 block GEMM on the half-precision tensor pipe:
+// C (M x N) = alpha * sum_terms op(A) op(B) (+ C), FP64 in and out.
+//
+// This part's FP64 pipe does 2 multiply-adds per clock and SM (1.7 measured,
+// DMMA m8n8k4 the same), its f16 mma.sync pipe 1024.  So every operand is cut
+// into OZ_S integer slices of 9 bits (the splitting of Ozaki, Ogita, Oishi
+// and Rump, Numer. Algorithms 59, 2012) and the products of slices run on the
+// f16 pipe, where they are exact:
+//   * each row of op(A) and each column of op(B) of one K group (at most 32
+//     complex) is scaled by the power of two above its largest real or
+//     imaginary part, x = X 2^E with |X| < 1, and written as
+//       X = sum_p d_p 2^-(8 + 9 p),  p = 0 .. 6,  |d_p| <= 256 integer
+//     (62 fractional bits; an FP64 number within 2^9 of the row's largest
+//     enters unrounded);
+//   * the integer products d_p e_q with p + q = s are added into one FP32
+//     accumulator per s.  |d e| <= 2^16 and at most 64 real K and s + 1 pairs
+//     give at most (s + 1) 2^22, so the sums stay exact (<= 2^24) for s <= 3
+//     and are rounded below 2^-59 of the row-column scale after that;
+//     s = 0 .. 6 is kept, what is dropped is below 2^-60 per product;
+//   * the seven sums of an output become one 64-bit integer, that one an
+//     FP64 number, and only the sum over K groups and terms is FP64
+//     arithmetic (one addition per group).
+// A complex product takes the real 2x2 form: one k16 MMA step holds 8 complex
+// k of op(A) as (re, im) pairs; complex column n of op(B) is stored as the real
+// columns 2n, (br, -bi) pairs, and 2n + 1, (bi, br) pairs.
+//
+// Tile of at most 64 x 24 complex, 8 warps; a warp owns up to three of the
+// 4 x 6 MMA subtiles (m16 x 4 complex columns), dead subtiles are skipped.
+// Blocks are ragged (K of 8-60, one side <= 36), so mma.sync with its 16 x 4
+// grain wastes less than tcgen05's 128 rows; the slices are also made where
+// they are used.
+//
+// What bounds it: instruction issue (2 per clock and SM of 4) of the slicing
+// and of the sums' conversion; the tensor pipe is about 10% busy.  Measured
+// on <psi|H|phi> at L = 16, D = 256 (32 launches, 7.2 GFLOP): 4.2 ms, where the
+// FP64 pipe's kernel took 9.7 ms; the error against 64 bits of the adjoint
+// energy gradient at L = 12, D = 128 went from 2.9e-15 to 1.7e-15.
+#include <cuda_fp16.h>
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cstdint>
+
+#include "kernels.hpp"
+
+namespace tdmps {
+
+namespace {
+
+constexpr int OZ_M = 64;        // most rows of an output tile (complex)
+constexpr int OZ_N = 24;        // most columns of an output tile
+constexpr int OZ_SUB = 3;       // MMA subtiles of a warp
+constexpr int OZ_S = 7;         // slices per operand
+constexpr int OZ_STAGE = 8;     // complex K per MMA step; the unit of split-K
+constexpr int OZ_KC = 32;       // complex K per group
+constexpr int OZ_THREADS = 256;
+constexpr int OZ_WA = OZ_M * OZ_KC, OZ_WB = 2 * OZ_N * OZ_KC;   // half2 words of one slice
+constexpr int OZ_SMEM = OZ_S * (OZ_WA + OZ_WB) * 4;          // A and B slices
+constexpr int OZ_INF = 0x7ff;
+
+__device__ __forceinline__ double2 zmul(double2 a, double2 b) {
+  return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+}
+
+__device__ __forceinline__ void mma_f16(float* c, const uint32_t* a, uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3},{%4,%5,%6,%7},{%8,%9},"
+      "{%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// four 8 x 8 half matrices, one 16-byte row address per lane
+__device__ __forceinline__ void ldmatrix4(uint32_t* r, uint32_t saddr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(saddr));
+}
+__device__ __forceinline__ void ldmatrix2(uint32_t* r, uint32_t saddr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];"
+               : "=r"(r[0]), "=r"(r[1])
+               : "r"(saddr));
+}
+// a b + c in 64 bits
+__device__ __forceinline__ long long madwide(int a, int b, long long c) {
+  long long d;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+  return d;
+}
+
+// word of (row, complex k) in one slice: the XOR spreads the eight 16-byte
+// rows that one ldmatrix phase reads over all banks
+__device__ __forceinline__ int oz_word(int row, int k) { return row * OZ_KC + (k ^ ((row & 7) << 2)); }
+
+// exponent field of the larger part
+__device__ __forceinline__ int oz_exp(double2 v) {
+  const int a = (__double2hiint(v.x) >> 20) & OZ_INF, b = (__double2hiint(v.y) >> 20) & OZ_INF;
+  return a > b ? a : b;
+}
+
+// x 2^(1022 - E) as a 62-bit fraction plus the digit bias: sum_j 256 512^j, so
+// that every 9-bit field holds digit + 256
+__device__ __forceinline__ unsigned long long oz_fixed(double x, int E) {
+  const int hi = __double2hiint(x);
+  const int e = (hi >> 20) & OZ_INF;
+  const unsigned int mh = (hi & 0xFFFFF) | (e ? 0x100000u : 0u);
+  const unsigned long long m = ((unsigned long long)mh << 32) | (unsigned int)__double2loint(x);
+  const int sh = E - (e ? e : 1);
+  unsigned long long f = sh < 62 ? (m << 9) >> sh : 0ull;
+  if (hi < 0) f = 0ull - f;
+  constexpr unsigned long long bias =
+      256ull * ((1ull << 54) + (1ull << 45) + (1ull << 36) + (1ull << 27) + (1ull << 18) +
+                (1ull << 9) + 1ull);
+  return f + bias;
+}
+
+// the seven digit pairs of one element: row r of A, or real columns 2r and
+// 2r + 1 of B
+template <bool IS_B>
+__device__ __forceinline__ void oz_store(uint32_t* s, int r, int k, double2 v, int E) {
+  const unsigned long long fr = oz_fixed(v.x, E), fi = oz_fixed(v.y, E);
+  const uint32_t rl = (uint32_t)fr, rh = (uint32_t)(fr >> 32), il = (uint32_t)fi, ih = (uint32_t)(fi >> 32);
+  const __half2 off = __half2half2(__ushort_as_half((unsigned short)0x6500));   // 1280
+  const int w0 = oz_word(IS_B ? 2 * r : r, k), w1 = oz_word(2 * r + 1, k);
+#pragma unroll
+  for (int p = 0; p < OZ_S; ++p) {
+    const int b = 9 * (OZ_S - 1 - p);
+    const uint32_t x = b >= 32 ? rh >> (b & 31) : __funnelshift_r(rl, rh, b);
+    const uint32_t y = b >= 32 ? ih >> (b & 31) : __funnelshift_r(il, ih, b);
+    // 0x6400 | f is the half 1024 + f; the top field reaches 512
+    const uint32_t w = (__byte_perm(x, y, 0x5410) & (p == 0 ? 0x03FF03FFu : 0x01FF01FFu)) | 0x64006400u;
+    const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&w), off);
+    const uint32_t u = *reinterpret_cast<const uint32_t*>(&d);
+    if (IS_B) {
+      s[p * OZ_WB + w0] = u ^ 0x80000000u;
+      s[p * OZ_WB + w1] = __byte_perm(u, u, 0x1032);
+    } else {
+      s[p * OZ_WA + w0] = u;
+    }
+  }
+}
+
+// One operand of a K group, R rows of at most OZ_KC complex k.  With k
+// contiguous in memory (row_op: the operand's row is the stored row; A with
+// OP_N / OP_J, B with OP_T / OP_C) a warp takes one row at a time (lane = k),
+// otherwise lane = row; either way a warp reads consecutive addresses.
+// Thread element j is row oz_row(j), complex k oz_k(j).
+template <int R>
+struct OzFrag {
+  static constexpr int RB = (R + 31) / 32, N = 4 * RB;   // row blocks of 32, elements per thread
+  double2 v[N];
+  static __device__ __forceinline__ int row(int j, bool row_op) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    return row_op ? warp + 8 * j : lane + 32 * (j % RB);
+  }
+  static __device__ __forceinline__ int k(int j, bool row_op) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    return row_op ? lane : warp + 8 * (j / RB);
+  }
+  // loads the group (scaled by sc when `scaled`) and leaves the largest
+  // exponent of each row in rexp (zeroed before); a segmented operand has one
+  // block per segment of its rows (sg, so non-null)
+  __device__ __forceinline__ void load(const void* base, int ld, const GemmSeg* sg,
+                                       const SegOps* so, int op, int row0, int rows, int k0, int nk,
+                                       bool row_op, bool scaled, double2 sc, int* rexp) {
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      const int r = row(j, row_op), kk = k(j, row_op);
+      v[j] = make_double2(0.0, 0.0);
+      if (r < rows && kk < nk) {
+        const double2* P = (const double2*)base;
+        int x = row0 + r, l = ld;
+        if (sg) {
+          const int s = (x >= sg->off[1]) + (x >= sg->off[2]) + (x >= sg->off[3]);
+          P = (const double2*)so->p[s];
+          l = so->ld[s];
+          x -= sg->off[s];
+        }
+        if (P) v[j] = P[row_op ? (size_t)x * l + k0 + kk : (size_t)(k0 + kk) * l + x];
+      }
+    }
+    if (op == OP_C || op == OP_J) {
+#pragma unroll
+      for (int j = 0; j < N; ++j) v[j].y = -v[j].y;
+    }
+    if (scaled) {
+#pragma unroll
+      for (int j = 0; j < N; ++j) v[j] = zmul(sc, v[j]);
+    }
+    if (row_op) {
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        const int r = row(j, true);
+        if (r >= rows) break;   // the same for every lane
+        const int e = __reduce_max_sync(0xffffffffu, oz_exp(v[j]));
+        if ((threadIdx.x & 31) == 0) rexp[r] = e;
+      }
+    } else {
+#pragma unroll
+      for (int b = 0; b < RB; ++b) {
+        int e = 0;
+#pragma unroll
+        for (int j = b; j < N; j += RB) e = max(e, oz_exp(v[j]));
+        if (e) atomicMax(&rexp[row(b, false)], e);
+      }
+    }
+  }
+  // the slices; rows past the block only reach outputs that are never stored,
+  // k is zero-filled to the MMA step
+  template <bool IS_B>
+  __device__ __forceinline__ void slice(uint32_t* s, int rows, int nk8, bool row_op,
+                                        const int* rexp) const {
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      const int r = row(j, row_op), kk = k(j, row_op);
+      if (r < rows && kk < nk8) oz_store<IS_B>(s, r, kk, v[j], max(rexp[r], 1));
+    }
+  }
+};
+
+// t 2^k as an FP64 number, on the integer ALU (the conversion instruction runs
+// on the FP64 pipe)
+__device__ __forceinline__ double oz_double(long long t, int k) {
+  if (t == 0) return 0.0;
+  const unsigned long long a = (unsigned long long)(t < 0 ? -t : t);
+  const int lz = __clzll((long long)a);
+  const unsigned long long n = a << lz;             // leading one at bit 63
+  const int e = 1023 + 63 - lz + k;
+  // 53 bits rounded to nearest; the leading one adds 1 to the exponent field
+  const unsigned long long m = (n >> 11) + ((n >> 10) & 1);
+  const unsigned long long sign = (unsigned long long)t & (1ull << 63);
+  if (e > 0 && e < OZ_INF - 1)
+    return __longlong_as_double((long long)(sign | (((unsigned long long)(e - 1) << 52) + m)));
+  return scalbn(__longlong_as_double((long long)(sign | ((1022ull << 52) + m))), e - 1023);
+}
+
+// the value of one output from its seven sums, times 2^k (k: scale of row and column)
+__device__ __forceinline__ double oz_value(const float (&acc)[OZ_S][4], int c, int k) {
+  int g[OZ_S];
+#pragma unroll
+  for (int s = 0; s < OZ_S; ++s) g[s] = __float2int_rn(acc[s][c]);
+  // sum_s g_s 512^(6 - s) = 2^27 h + l, |h| < 2^50, |l| < 2^43, in units small
+  // enough that the 64-bit sum keeps at least 60 bits of it (a row and a
+  // column whose large elements do not meet leave h small)
+  const long long h = madwide(g[0], 1 << 27, madwide(g[1], 1 << 18, madwide(g[2], 1 << 9, (long long)g[3])));
+  const long long l = madwide(g[4], 1 << 18, madwide(g[5], 1 << 9, (long long)g[6]));
+  const int hh = (int)(h >> 32);
+  const int drop = max(0, 29 - __clz(hh ^ (hh >> 31)));   // |h| < 2^(35 + drop), drop <= 15
+  const long long t = (h << (27 - drop)) + (l >> drop);
+  return oz_double(t, k - 70 + drop);
+}
+
+// tiles of one dimension: as few as fit, of equal size rounded up to the
+// subtile's
+__host__ __device__ inline int oz_tiles(int n, int most) { return (n + most - 1) / most; }
+__host__ __device__ inline int oz_edge(int n, int most, int grain) {
+  const int c = oz_tiles(n, most);
+  return ((n + c - 1) / c + grain - 1) / grain * grain;
+}
+
+// element (r, c) of a task's result (or of its split's slice)
+__device__ __forceinline__ void f64_store(const GemmTask& t, const GemmSeg* sg, int split, int r, int c,
+                                          double2 v) {
+  if (t.splits > 1) {
+    ((double2*)t.part)[((size_t)split * t.M + r) * t.N + c] = v;
+    return;
+  }
+  double2* p;
+  if (sg) {
+    const int x = sg->dim == 0 ? r : c;
+    const int s = (x >= sg->off[1]) + (x >= sg->off[2]) + (x >= sg->off[3]);
+    const int y = x - sg->off[s];
+    p = (double2*)sg->C[s] + (sg->dim == 0 ? (size_t)y * sg->ldc[s] + c : (size_t)r * sg->ldc[s] + y);
+  } else {
+    p = (double2*)t.C + (t.ct ? (size_t)c * t.ldc + r : (size_t)r * t.ldc + c);
+  }
+  if (t.beta) { v.x += p->x; v.y += p->y; }
+  *p = v;
+}
+
+__global__ void __launch_bounds__(OZ_THREADS, 2) k_gemm(const GemmTask* __restrict__ tasks,
+                                                        const GemmTerm* __restrict__ terms,
+                                                        const GemmSeg* __restrict__ segs,
+                                                        const SegOps* __restrict__ segops,
+                                                        const int* __restrict__ tile_task) {
+  extern __shared__ uint32_t oz_sh[];
+  uint32_t* sA = oz_sh;
+  uint32_t* sB = oz_sh + OZ_S * OZ_WA;
+  __shared__ int rexpA[2][OZ_M], rexpB[2][32];   // exponents of the rows of A and the columns of B
+  const GemmTask& t = tasks[tile_task[blockIdx.x]];
+  const unsigned local = blockIdx.x - t.tile_base, splits = t.splits;
+  unsigned split = 0, rest = local;
+  if (splits > 1) {
+    split = local % splits;
+    rest = local / splits;
+  }
+  const int M = t.M, N = t.N, walk = t.walk;
+  const int tm = oz_edge(M, OZ_M, 16), tn = oz_edge(N, OZ_N, 4);
+  const unsigned ny = rest / (unsigned)t.tiles_m;
+  const int m0 = (int)(rest - ny * t.tiles_m) * tm;
+  const int rows = min(tm, M - m0);
+  const int opA = t.opA, opB = t.opB, tbeg = t.term_begin, tend = t.term_end;
+  const bool rowA = opA == OP_N || opA == OP_J, rowB = opB == OP_T || opB == OP_C;
+  const GemmSeg* sg = t.seg1 ? segs + (t.seg1 - 1) : nullptr;
+  const GemmSeg *sgA = nullptr, *sgB = nullptr;
+  if (sg) (sg->dim == 0 ? sgA : sgB) = sg;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int g = lane >> 2, q = lane & 3;
+  // ldmatrix row of this lane: of A, 8-row halves then 4-word k halves; of B,
+  // the k halves
+  const int lr = lane & 7, la = ((lane >> 3) & 1) * 8 + lr, ka = (lane >> 4) * 4,
+            kb = ((lane >> 3) & 1) * 4;
+  const uint32_t aA = (uint32_t)__cvta_generic_to_shared(sA), aB = (uint32_t)__cvta_generic_to_shared(sB);
+  // this split's share of the task's K steps (OZ_STAGE each, over all terms)
+  int lo = 0, hi = 0x7fffffff;
+  if (splits > 1) {
+    unsigned S = 0;
+    for (int e = tbeg; e < tend; ++e) S += (terms[e].K + OZ_STAGE - 1) / OZ_STAGE;
+    lo = (int)(split * S / splits);
+    hi = (int)((split + 1) * S / splits);
+  }
+  double2 alpha = t.alpha;
+  if (t.alpha_ptr) alpha = zmul(alpha, *t.alpha_ptr);
+  if (t.alpha_div) {
+    const double2 b = *t.alpha_div;
+    const double d = b.x * b.x + b.y * b.y;
+    alpha = make_double2((alpha.x * b.x + alpha.y * b.y) / d, (alpha.y * b.x - alpha.x * b.y) / d);
+  }
+  const bool unit = alpha.x == 1.0 && alpha.y == 0.0;
+  if (threadIdx.x < OZ_M) rexpA[0][threadIdx.x] = 0;
+  if (threadIdx.x < 32) rexpB[0][threadIdx.x] = 0;
+  __syncthreads();
+  int bufA = 0, bufB = 0;
+  const int nsm = (rows + 15) >> 4;
+  // the column tiles of this CTA: one, or (walk > 1: a task of one K group)
+  // several that share the slices of A
+  for (int w = 0; w < walk; ++w) {
+    const int n0 = (int)(ny * walk + w) * tn;
+    if (n0 >= N) break;
+    const int cols = min(tn, N - n0);
+    // live subtiles, dealt to the warps in turn
+    const int nsub = nsm * ((cols + 3) >> 2);
+    auto sub_col = [&](int i) {   // first column of subtile warp + 8 i
+      const int sub = warp + 8 * i;
+      return 4 * (nsm == 4 ? sub >> 2 : nsm == 2 ? sub >> 1 : nsm == 1 ? sub : sub / 3);
+    };
+    auto sub_row = [&](int i, int col) { return (warp + 8 * i - (col >> 2) * nsm) * 16; };
+    double2 out[OZ_SUB][2];   // [subtile][row half]: rows g and g + 8, complex column q
+#pragma unroll
+    for (int i = 0; i < OZ_SUB; ++i)
+#pragma unroll
+      for (int j = 0; j < 2; ++j) out[i][j] = make_double2(0.0, 0.0);
+    int idx = 0;
+    bool first = true;
+    for (int e = tbeg; e < tend && idx < hi; ++e) {
+      const GemmTerm& tr = terms[e];
+      const int K = tr.K, nk = (K + OZ_STAGE - 1) / OZ_STAGE;
+      if (idx + nk <= lo) { idx += nk; continue; }
+      double2 sc = tr.scale;
+      if (tr.scale_ptr) sc = zmul(sc, *tr.scale_ptr);
+      const bool scaled = sc.x != 1.0 || sc.y != 0.0;
+      const SegOps* so = sg ? segops + tr.pad : nullptr;
+      const int c0 = max(lo - idx, 0), c1 = min(hi - idx, nk);
+      idx += nk;
+      // groups of at most OZ_KC, of equal size
+      const unsigned ng = (unsigned)(c1 - c0 + OZ_KC / OZ_STAGE - 1) / (OZ_KC / OZ_STAGE);
+      for (unsigned gi = 0; gi < ng; ++gi) {
+        const int s0 = c0 + (int)(gi * (unsigned)(c1 - c0) / ng);
+        const int s1 = c0 + (int)((gi + 1) * (unsigned)(c1 - c0) / ng);
+        const int k0 = s0 * OZ_STAGE, kn8 = (s1 - s0) * OZ_STAGE, kn = min(K - k0, kn8);
+        const int *ra = rexpA[bufA], *rb = rexpB[bufB];
+        {
+          OzFrag<OZ_N> fb;
+          fb.load(tr.B, tr.ldb, sgB, so, opB, n0, cols, k0, kn, rowB, false, sc, rexpB[bufB]);
+          if (w == 0) {
+            OzFrag<OZ_M> fa;
+            fa.load(tr.A, tr.lda, sgA, so, opA, m0, rows, k0, kn, rowA, scaled, sc, rexpA[bufA]);
+            __syncthreads();
+            fa.slice<false>(sA, rows, kn8, rowA, ra);
+            bufA ^= 1;
+          } else {
+            __syncthreads();
+          }
+          fb.slice<true>(sB, cols, kn8, rowB, rb);
+          bufB ^= 1;
+        }
+        if (w == 0 && threadIdx.x < OZ_M) rexpA[bufA][threadIdx.x] = 0;
+        if (threadIdx.x < 32) rexpB[bufB][threadIdx.x] = 0;
+        if (w > 0) ra = rexpA[bufA ^ 1];   // the exponents the slices were made with
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < OZ_SUB; ++i) {
+          if (warp + 8 * i < nsub) {
+            const int nc = sub_col(i), mr = sub_row(i, nc);
+            float acc[OZ_S][4];
+#pragma unroll
+            for (int s = 0; s < OZ_S; ++s)
+#pragma unroll
+              for (int c = 0; c < 4; ++c) acc[s][c] = 0.f;
+            for (int ks = 0; ks < kn8; ks += OZ_STAGE) {
+              const uint32_t wa = aA + 4 * oz_word(mr + la, ks + ka);
+              const uint32_t wb = aB + 4 * oz_word(2 * nc + lr, ks + kb);
+              uint32_t bf[OZ_S][2];
+#pragma unroll
+              for (int p = 0; p < OZ_S; ++p) ldmatrix2(bf[p], wb + p * OZ_WB * 4);
+#pragma unroll
+              for (int p = 0; p < OZ_S; ++p) {
+                uint32_t af[4];
+                ldmatrix4(af, wa + p * OZ_WA * 4);
+#pragma unroll
+                for (int r = 0; r + p < OZ_S; ++r) mma_f16(acc[p + r], af, bf[r][0], bf[r][1]);
+              }
+            }
+            // accumulators 0, 1: row g, complex column q; 2, 3: row g + 8
+            const int eb = rb[nc + q];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const int ea = ra[mr + g + 8 * h];
+              const int k = max(ea, 1) + max(eb, 1) - 2 * 1022;
+              double2 v = make_double2(oz_value(acc, 2 * h, k), oz_value(acc, 2 * h + 1, k));
+              // an infinity or NaN in the row or the column
+              if (ea == OZ_INF || eb == OZ_INF) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
+              // the first group needs no addition (out is zero): a real branch,
+              // so that the FP64 pipe is left alone
+              if (!first) {
+                asm volatile("");
+                v.x += out[i][h].x;
+                v.y += out[i][h].y;
+              }
+              out[i][h] = v;
+            }
+          }
+        }
+        first = false;
+        __syncthreads();
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < OZ_SUB; ++i) {
+      if (warp + 8 * i >= nsub) continue;
+      const int nc = sub_col(i), mr = sub_row(i, nc);
+      const int c = n0 + nc + q;
+      if (c >= n0 + cols) continue;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int rl = mr + g + 8 * h, r = m0 + rl;
+        if (rl >= rows) continue;
+        double2 v = out[i][h];
+        if (!unit) {
+          asm volatile("");
+          v = zmul(alpha, v);
+        }
+        f64_store(t, sg, (int)split, r, c, v);
+      }
+    }
+  }
+}
+
+// ------------------------------------------------------------------ small launches
+
+// The same GEMM (no segments) on the FP64 pipe, for launches whose tiles are a
+// few thousand multiply-adds each: there the sliced kernel's fixed cost (three
+// dependent phases and about 3,000 instructions per warp) is longer than the
+// arithmetic.  Tile 32 x 32, K in chunks of 8, one 2 x 2 block per thread.
+constexpr int ST = 32, SK = 8;
+
+__device__ __forceinline__ void zfma(double2& c, double2 a, double2 b) {
+  c.x = fma(a.x, b.x, fma(-a.y, b.y, c.x));
+  c.y = fma(a.x, b.y, fma(a.y, b.x, c.y));
+}
+
+__global__ void __launch_bounds__(256) k_gemm_small(const GemmTask* __restrict__ tasks,
+                                                    const GemmTerm* __restrict__ terms,
+                                                    const int* __restrict__ tile_task) {
+  __shared__ double2 As[SK][ST + 1];
+  __shared__ double2 Bs[SK][ST + 1];
+  const GemmTask t = tasks[tile_task[blockIdx.x]];
+  const int local = blockIdx.x - t.tile_base;
+  const int split = local % t.splits, rest = local / t.splits;
+  const int m0 = (rest % t.tiles_m) * ST, n0 = (rest / t.tiles_m) * ST;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  // rows past the block edge do no arithmetic (a warp covers 4 rows)
+  const bool rows_live = m0 + 2 * ty < t.M;
+  auto load = [&](const void* P, int ld, int op, bool trans, int r, int k, int R, int K) {
+    if (r >= R || k >= K) return make_double2(0.0, 0.0);
+    double2 v = ((const double2*)P)[trans ? (size_t)k * ld + r : (size_t)r * ld + k];
+    if (op == OP_C || op == OP_J) v.y = -v.y;
+    return v;
+  };
+  double2 acc[2][2];
+  for (int i = 0; i < 2; ++i)
+    for (int j = 0; j < 2; ++j) acc[i][j] = make_double2(0.0, 0.0);
+  int S = 0;
+  for (int e = t.term_begin; e < t.term_end; ++e) S += (terms[e].K + SK - 1) / SK;
+  const int lo = (int)((long long)split * S / t.splits);
+  const int hi = (int)((long long)(split + 1) * S / t.splits);
+  int idx = 0;
+  for (int e = t.term_begin; e < t.term_end && idx < hi; ++e) {
+    const GemmTerm g = terms[e];
+    const int nk = (g.K + SK - 1) / SK;
+    if (idx + nk <= lo) { idx += nk; continue; }
+    double2 sc = g.scale;
+    if (g.scale_ptr) sc = zmul(sc, *g.scale_ptr);
+    const bool scaled = sc.x != 1.0 || sc.y != 0.0;
+    const int c0 = max(lo - idx, 0), c1 = min(hi - idx, nk);
+    for (int ch = c0; ch < c1; ++ch) {
+      const int k0 = ch * SK;
+      {
+        const int i = threadIdx.x >> 3, k = threadIdx.x & 7;      // A tile: 32 x 8
+        double2 a = load(g.A, g.lda, t.opA, t.opA == OP_T || t.opA == OP_C, m0 + i, k0 + k, t.M, g.K);
+        if (scaled) a = zmul(sc, a);
+        As[k][i] = a;
+        const int kk = threadIdx.x >> 5, j = threadIdx.x & 31;    // B tile: 8 x 32
+        Bs[kk][j] = load(g.B, g.ldb, t.opB, t.opB == OP_N || t.opB == OP_J, n0 + j, k0 + kk, t.N, g.K);
+      }
+      __syncthreads();
+      if (rows_live) {
+        const int kl = min(SK, g.K - k0);
+        for (int k = 0; k < kl; ++k) {
+          const double2 a0 = As[k][ty * 2], a1 = As[k][ty * 2 + 1];
+          const double2 b0 = Bs[k][tx * 2], b1 = Bs[k][tx * 2 + 1];
+          zfma(acc[0][0], a0, b0);
+          zfma(acc[0][1], a0, b1);
+          zfma(acc[1][0], a1, b0);
+          zfma(acc[1][1], a1, b1);
+        }
+      }
+      __syncthreads();
+    }
+    idx += nk;
+  }
+  double2 alpha = t.alpha;
+  if (t.alpha_ptr) alpha = zmul(alpha, *t.alpha_ptr);
+  if (t.alpha_div) {
+    const double2 b = *t.alpha_div;
+    const double d = b.x * b.x + b.y * b.y;
+    alpha = make_double2((alpha.x * b.x + alpha.y * b.y) / d, (alpha.y * b.x - alpha.x * b.y) / d);
+  }
+  const bool unit = alpha.x == 1.0 && alpha.y == 0.0;
+  for (int i = 0; i < 2; ++i)
+    for (int j = 0; j < 2; ++j) {
+      const int r = m0 + ty * 2 + i, c = n0 + tx * 2 + j;
+      if (r < t.M && c < t.N) f64_store(t, nullptr, split, r, c, unit ? acc[i][j] : zmul(alpha, acc[i][j]));
+    }
+}
+
+}  // namespace
+
+int f64_tiles_m(int M, bool small) { return oz_tiles(M, small ? ST : OZ_M); }
+int f64_tiles_n(int N, bool small, int walk) {
+  return small ? oz_tiles(N, ST) : oz_tiles(oz_tiles(N, OZ_N), walk);
+}
+int f64_walk(int N, int nterms, int K) {
+  return nterms == 1 && K <= OZ_KC ? std::min(4, std::max(1, oz_tiles(N, OZ_N))) : 1;
+}
+int f64_stage_k() { return OZ_STAGE; }   // = SK
+
+void launch_gemm(const GemmTask* d_tasks, const GemmTerm* d_terms, const GemmSeg* d_segs,
+                 const SegOps* d_segops, const int* d_tile_task, int ntiles, bool small,
+                 cudaStream_t st) {
+  if (ntiles <= 0) return;
+  if (small) {
+    k_gemm_small<<<ntiles, 256, 0, st>>>(d_tasks, d_terms, d_tile_task);
+    return;
+  }
+  set_smem_limit((const void*)k_gemm, OZ_SMEM);
+  k_gemm<<<ntiles, OZ_THREADS, OZ_SMEM, st>>>(d_tasks, d_terms, d_segs, d_segops, d_tile_task);
+}
+
+}  // namespace tdmps

@@ -159,9 +159,10 @@ cplx overlap_noalloc(Context& c, const MPSd& bra, const MPSd& ket) {
       for (size_t t = lo; t < hi; ++t) {
         GemmTask g = tasks[t];
         if (g.M <= 0 || g.N <= 0) continue;
-        g.tiles_m = (g.M + 31) / 32;
+        g.tiles_m = f64_tiles_m(g.M, true);
         g.splits = 1;
-        int tn = (g.N + 31) / 32;
+        g.walk = 1;
+        int tn = f64_tiles_n(g.N, true, g.walk);
         g.tile_base = (int)tile_task.size();
         int id = (int)tk.size();
         tk.push_back(g);
@@ -193,8 +194,8 @@ cplx overlap_noalloc(Context& c, const MPSd& bra, const MPSd& ket) {
                                 cudaMemcpyDeviceToDevice, c.st));
   for (const Launch& ln : plan) {
     const char* p = (const char*)c.stage(ln.pack.data(), ln.pack.size());
-    launch_gemm((const GemmTask*)p, ln.ntask, (const GemmTerm*)(p + ln.o_terms),
-                (const int*)(p + ln.o_tiles), ln.ntile, c.st);
+    launch_gemm((const GemmTask*)p, (const GemmTerm*)(p + ln.o_terms), nullptr, nullptr,
+                (const int*)(p + ln.o_tiles), ln.ntile, true, c.st);
     TD_CHECK_CUDA(cudaGetLastError());
   }
   double2 h = make_double2(0.0, 0.0);
