@@ -753,342 +753,284 @@ void launch_svd(const FactTask* d_tasks, int ntasks, int* d_status, cudaStream_t
 
 // ------------------------------------------------------------------ Gram-Schmidt QR
 
-// Classical Gram-Schmidt with re-orthogonalisation on a column-major m x n
-// matrix.  The second projection pass runs when the first one removed more
-// than 1 - 1/sqrt(2) of the column's norm (the Daniel-Gragg-Kaufman-Stewart
-// criterion: otherwise one classical pass is already orthogonal to working
-// precision); it halves the FP64 work on well-conditioned blocks.  Columns
-// whose residual norm falls to <= 1e-12 times the largest input column norm
-// are dependent: they add no new direction (such a column always lost far
-// more than the criterion's share, so it always gets both passes).  The
-// independent directions are stored compactly in the first columns (at most
-// k = min(m, n)), the remaining of the first k columns are zero.  R (k x n,
-// column-major, leading dimension n) holds the coefficients, so that
-// A = Q R.
-constexpr int QR_THREADS = 256;
-constexpr int QR_SMEM = 200 * 1024;   // matrix held in shared memory when it fits
+// Modified Gram-Schmidt with conditional re-orthogonalisation on column-major
+// m x n matrices: A = Q R, one matrix per cluster of CS CTAs (CS = 1: one CTA).
+// CTA `rank` holds rows [rank*mc, rank*mc + mc), in shared memory when they
+// fit, else in place in global memory.
+//
+// Right-looking: at step j the pivot v = a_j (already orthogonal to the
+// accepted columns) is multiplied with every remaining column at once,
+//   p_c = v^H a_c (c >= j; p_j = |v|^2),   a_c -= v p_c / p_j,
+// so a step is one set of independent inner products, one cluster reduction
+// and one rank-one update; nothing is summed serially over the earlier
+// columns, and roots and the normalisation wait until the end (the FP64 pipe
+// does two multiply-adds per clock and SM, so serial chains and work repeated
+// on every lane are what costs here).  Each CTA writes its partial products
+// into a slot of every CTA, the cluster barrier publishes them, and every CTA
+// adds the slots in rank order: all hold the same bits and take the same
+// branches.  Slots are double buffered: the barrier of reduction r also tells
+// a CTA that every CTA has read the buffer of reduction r - 1.
+//
+// A column that lost more than half of its squared norm to the earlier ones
+// (the Daniel-Gragg-Kaufman-Stewart criterion, on norms down-dated by
+// |p_c|^2 / p_j) is projected once more against all accepted columns before
+// it becomes the pivot.  A column whose residual norm is <= 1e-12 times the
+// largest input column norm adds no direction.  Accepted directions are
+// stored compactly in the first columns (at most k = min(m, n)), the others
+// of the first k columns are zero.  R (n x n, column-major) holds the
+// coefficients.
+//
+// Measured (one fitted H|psi>, L = 16, D = 256: 45 launches of ~38 sectors, n up
+// to 25): 3.5 ms, where a left-looking form with five to seven block barriers
+// and serial sums per column took 8.75 ms.  256 threads: 3.6 ms, 512: 4.2 ms;
+// clusters of 4 CTAs: 3.5 ms.
+constexpr int QR_THREADS = 128;
+constexpr int QR_CS = 8;
+constexpr double QR_CLUSTER_WORK = 12000;   // m n^2 from which a matrix gets a cluster
+constexpr int QR_SMEM = 200 * 1024;
+constexpr int QR_BATCH = 512;         // columns of one reduction
+constexpr int QR_BATCH_GLOBAL = 256;  // the same when the matrix stays in global memory
 
-__global__ void __launch_bounds__(QR_THREADS) k_qr(const FactTask* __restrict__ tasks) {
-  extern __shared__ double2 sh[];
-  const FactTask t = tasks[blockIdx.x];
-  const int m = t.m, n = t.n, kmax = m < n ? m : n;
-  // layout: [v: m][coef: n][A: m*n][R: n*n] when they fit
-  double2* v = sh;
-  double2* coef = sh + m;
-  const bool a_sh =
-      (size_t)(m + n + (size_t)m * n + (size_t)n * n) * sizeof(double2) <= (size_t)QR_SMEM;
-  double2* A = a_sh ? sh + m + n : t.A;
-  double2* R = a_sh ? sh + m + n + (size_t)m * n : t.V;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-  __shared__ double maxn, vn, vinv;
-  __shared__ int nq;
-  if (threadIdx.x == 0) { maxn = 0.0; nq = 0; }
-  if (a_sh)
-    for (size_t e = threadIdx.x; e < (size_t)m * n; e += blockDim.x) A[e] = t.A[e];
-  for (int e = threadIdx.x; e < n * n; e += blockDim.x) R[e] = make_double2(0.0, 0.0);
-  __syncthreads();
-  for (int j = warp; j < n; j += nwarp) {
-    double s2 = 0.0;
-    for (int i = lane; i < m; i += 32) s2 += cabs2(A[(size_t)j * m + i]);
-    s2 = warp_sum(s2);
-    if (lane == 0) {
-      // non-negative doubles order like their bit patterns
-      atomicMax((unsigned long long*)&maxn, (unsigned long long)__double_as_longlong(sqrt(s2)));
-    }
-  }
-  __syncthreads();
-  const double tol = 1e-12 * maxn;
-  for (int j = 0; j < n; ++j) {
-    for (int i = threadIdx.x; i < m; i += blockDim.x) v[i] = A[(size_t)j * m + i];
-    __syncthreads();
-    const int q = nq;
-    double norm_before = 0.0;
-    if (q > 0 && warp == 0) {
-      double s2 = 0.0;
-      for (int i = lane; i < m; i += 32) s2 += cabs2(v[i]);
-      s2 = warp_sum(s2);
-      if (lane == 0) vn = s2;
-    }
-    if (q > 0) {
-      __syncthreads();
-      norm_before = vn;
-    }
-    for (int pass = 0; pass < 2 && q > 0; ++pass) {
-      for (int cc = warp; cc < q; cc += nwarp) {
-        const double2* qc = A + (size_t)cc * m;
-        double re = 0.0, im = 0.0;
-        for (int i = lane; i < m; i += 32) {
-          double2 a = qc[i], b = v[i];
-          re += a.x * b.x + a.y * b.y;   // conj(q) * v
-          im += a.x * b.y - a.y * b.x;
-        }
-        re = warp_sum(re); im = warp_sum(im);
-        if (lane == 0) coef[cc] = make_double2(re, im);
-      }
-      __syncthreads();
-      for (int i = threadIdx.x; i < m; i += blockDim.x) {
-        double2 acc = v[i];
-        for (int cc = 0; cc < q; ++cc) acc = csub(acc, cmul(coef[cc], A[(size_t)cc * m + i]));
-        v[i] = acc;
-      }
-      for (int cc = threadIdx.x; cc < q; cc += blockDim.x) {
-        double2* rr = R + (size_t)j * n + cc;   // R[c, j], leading dimension n
-        *rr = cadd(*rr, coef[cc]);
-      }
-      __syncthreads();
-      if (pass == 0) {
-        if (warp == 0) {
-          double s2 = 0.0;
-          for (int i = lane; i < m; i += 32) s2 += cabs2(v[i]);
-          s2 = warp_sum(s2);
-          if (lane == 0) vn = s2;
-        }
-        __syncthreads();
-        const bool again = vn < 0.5 * norm_before;   // |v'|^2 < |v|^2 / 2
-        __syncthreads();
-        if (!again) break;
-      }
-    }
-    if (warp == 0) {
-      double s2 = 0.0;
-      for (int i = lane; i < m; i += 32) s2 += cabs2(v[i]);
-      s2 = warp_sum(s2);
-      if (lane == 0) {
-        vn = sqrt(s2);
-        vinv = vn > 0.0 ? 1.0 / vn : 0.0;   // once, not on every thread (FP64 pipe)
-      }
-    }
-    __syncthreads();
-    const double nrm = vn;
-    if (nrm > tol && q < kmax) {
-      const double inv = vinv;
-      for (int i = threadIdx.x; i < m; i += blockDim.x) A[(size_t)q * m + i] = cscale(v[i], inv);
-      if (threadIdx.x == 0) {
-        R[(size_t)j * n + q] = make_double2(nrm, 0.0);
-        nq = q + 1;
-      }
-    }
-    __syncthreads();
-  }
-  const int nfin = nq;
-  for (int cc = nfin; cc < kmax; ++cc)
-    for (int i = threadIdx.x; i < m; i += blockDim.x) A[(size_t)cc * m + i] = make_double2(0.0, 0.0);
-  if (a_sh) {
-    __syncthreads();
-    for (size_t e = threadIdx.x; e < (size_t)m * kmax; e += blockDim.x) t.A[e] = A[e];
-    for (size_t e = threadIdx.x; e < (size_t)n * n; e += blockDim.x) t.V[e] = R[e];
-  }
+__host__ __device__ inline int qr_mc(int m, int cs) { return (m + cs - 1) / cs; }
+// complex elements of dynamic shared memory: slots, factors, squared pivots
+// and column norms, projection partials; then the rows
+__host__ __device__ inline size_t qr_fixed(int n, int cs, int batch) {
+  const size_t nb = n < batch ? n : batch;
+  return 2 * (size_t)cs * nb + nb + (3 * (size_t)n + 1) / 2 + ((size_t)n + 3) / 4 + 1 + QR_THREADS;
 }
 
-// The same Gram-Schmidt QR (dependency rule, conditional second pass)
-// with one sector spread over a cluster of QRC_CS CTAs: CTA `rank` holds
-// rows [rank*mc, rank*mc + mc) of the matrix in its shared memory, and every
-// inner product (projection coefficients, norms) is a partial sum per CTA
-// combined across the cluster through distributed shared memory.  Each CTA
-// writes its partial vector into a slot of every CTA, the cluster barrier
-// publishes them, and every CTA adds the slots in rank order -- so all CTAs
-// hold bit-identical sums and take identical branch decisions.  Slots are
-// double buffered: the barrier of reduction r also tells a CTA that every
-// CTA has read the buffer of reduction r - 1, which reduction r + 1 reuses.
-// A sector's FP64 work is divided by the cluster size, which is what limits
-// the single-CTA kernel on large sectors (one SM's FP64 pipe).
-constexpr int QRC_CS = 8;
-constexpr int QRC_THREADS = 256;
-
-__host__ __device__ inline int qrc_mc(int m) { return (m + QRC_CS - 1) / QRC_CS; }
-// complex elements of dynamic shared memory per CTA
-__host__ __device__ inline size_t qrc_elems(int m, int n) {
-  const size_t mc = qrc_mc(m);
-  return mc * n + mc + n + 2 * (size_t)QRC_CS * (n + 1) + 8;
-}
-
-__global__ void __launch_bounds__(QRC_THREADS) k_qr_cl(const FactTask* __restrict__ tasks) {
+template <int CS>
+__global__ void __launch_bounds__(QR_THREADS) k_qr(const FactTask* __restrict__ tasks, int batch,
+                                                   int smem_elems) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
-  extern __shared__ double2 shc[];
-  const int rank = (int)cl.block_rank();
-  const FactTask t = tasks[blockIdx.x / QRC_CS];
+  extern __shared__ double2 qr_sh[];
+  const int rank = CS > 1 ? (int)cl.block_rank() : 0;
+  const FactTask t = tasks[blockIdx.x / CS];
   const int m = t.m, n = t.n, kmax = m < n ? m : n;
-  const int mc = qrc_mc(m);
-  const int row0 = rank * mc;
+  const int mc = qr_mc(m, CS), row0 = rank * mc;
   const int ml = max(0, min(mc, m - row0));   // rows held here
-  const int SL = n + 1;                       // slot length
-  double2* A = shc;                           // [n][mc]
-  double2* v = A + (size_t)mc * n;            // [mc]
-  double2* coef = v + mc;                     // [n]
-  double2* slots = coef + n;                  // [2][CS][SL]
-  double2* scal = slots + 2 * (size_t)QRC_CS * SL;   // small scratch
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+  const int NB = n < batch ? n : batch;
+  double2* slots = qr_sh;                        // [2][CS][NB]
+  double2* fac = slots + 2 * (size_t)CS * NB;    // [NB]
+  double2* pp = fac + NB;                        // [QR_THREADS]
+  double* piv = (double*)(pp + QR_THREADS);      // [n] squared norms of the accepted columns
+  double* orig = piv + n;                        // [n] squared column norms
+  double* est = orig + n;                        // [n] the same, down-dated
+  int* again = (int*)(est + n);                  // [n] the column needs the second projection
+  __shared__ int keep_sh;
+  const size_t fixed = qr_fixed(n, CS, batch);
+  const bool a_sh = fixed + (size_t)mc * n <= (size_t)smem_elems;
+  double2* A = a_sh ? qr_sh + fixed : t.A + row0;   // column c at A + c * lda
+  const size_t lda = a_sh ? mc : m;
+  const int tid = threadIdx.x;
   int red = 0;
-  // all-reduce of len values (mine may alias out)
-  auto allreduce = [&](const double2* mine, int len, double2* out) {
-    const int buf = red & 1;
+
+  // partial products conj(x) . y of the local rows for the columns [c0, c0 + cnt),
+  // 1 to 8 lanes per column, into this CTA's slot of every CTA; then the barrier.
+  // self: |a_c|^2 of each column, else column x times column c
+  auto products = [&](const double2* x, int c0, int cnt, bool self) {
+    const int lpc = cnt * 8 <= QR_THREADS ? 8 : cnt * 4 <= QR_THREADS ? 4 : cnt * 2 <= QR_THREADS ? 2 : 1;
+    const int sub = tid & (lpc - 1), step = QR_THREADS / lpc;
+    const int b = red & 1;
+    // every lane of a warp takes part in the shuffles
+    for (int k0 = 0; k0 < cnt; k0 += step) {
+      const int k = k0 + tid / lpc;
+      double re = 0.0, im = 0.0;
+      if (k < cnt) {
+        const double2* y = A + (size_t)(c0 + k) * lda;
+        const double2* p = self ? y : x;
+        for (int i = sub; i < ml; i += lpc) {
+          const double2 u = p[i], w = y[i];
+          re = fma(u.x, w.x, fma(u.y, w.y, re));
+          im = fma(u.x, w.y, fma(-u.y, w.x, im));
+        }
+      }
+      for (int o = lpc >> 1; o > 0; o >>= 1) {
+        re += __shfl_xor_sync(0xffffffffu, re, o);
+        im += __shfl_xor_sync(0xffffffffu, im, o);
+      }
+      if (k < cnt)
+        for (int r = sub; r < CS; r += lpc) {
+          double2* dst = CS > 1 ? cl.map_shared_rank(slots, r) : slots;
+          dst[((size_t)b * CS + rank) * NB + k] = make_double2(re, im);
+        }
+    }
+    if (CS > 1) cl.sync(); else __syncthreads();
     ++red;
-    for (int r = 0; r < QRC_CS; ++r) {
-      double2* dst = cl.map_shared_rank(slots, r) + ((size_t)buf * QRC_CS + rank) * SL;
-      for (int i = threadIdx.x; i < len; i += blockDim.x) dst[i] = mine[i];
-    }
-    cl.sync();
-    for (int i = threadIdx.x; i < len; i += blockDim.x) {
-      double2 acc = make_double2(0.0, 0.0);
-      for (int r = 0; r < QRC_CS; ++r) acc = cadd(acc, slots[((size_t)buf * QRC_CS + r) * SL + i]);
-      out[i] = acc;
-    }
-    __syncthreads();
   };
-  // squared norm of v over all rows
-  auto vnorm2 = [&]() {
-    if (warp == 0) {
-      double s2 = 0.0;
-      for (int i = lane; i < ml; i += 32) s2 += cabs2(v[i]);
-      s2 = warp_sum(s2);
-      if (lane == 0) scal[0] = make_double2(s2, 0.0);
-    }
-    __syncthreads();
-    allreduce(scal, 1, scal + 1);
-    return scal[1].x;
+  // entry k of the last reduction
+  auto total = [&](int k) {
+    const double2* s = slots + (size_t)((red - 1) & 1) * CS * NB + k;
+    double2 v = s[0];
+#pragma unroll
+    for (int r = 1; r < CS; ++r) v = cadd(v, s[(size_t)r * NB]);
+    return v;
   };
 
-  for (int c = 0; c < n; ++c)
-    for (int i = threadIdx.x; i < ml; i += blockDim.x) A[(size_t)c * mc + i] = t.A[(size_t)c * m + row0 + i];
+  if (a_sh)
+    for (int c = tid >> 5; c < n; c += QR_THREADS / 32)
+      for (int i = tid & 31; i < ml; i += 32) A[c * lda + i] = t.A[(size_t)c * m + row0 + i];
   if (rank == 0)
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) t.V[e] = make_double2(0.0, 0.0);
-  // the rows were staged by every thread; each warp reads whole columns
+    for (int e = tid; e < n * n; e += QR_THREADS) t.V[e] = make_double2(0.0, 0.0);
   __syncthreads();
-  // largest column norm
-  for (int c = warp; c < n; c += nwarp) {
-    double s2 = 0.0;
-    for (int i = lane; i < ml; i += 32) s2 += cabs2(A[(size_t)c * mc + i]);
-    s2 = warp_sum(s2);
-    if (lane == 0) coef[c] = make_double2(s2, 0.0);
+  for (int c0 = 0; c0 < n; c0 += NB) {
+    const int cnt = min(NB, n - c0);
+    products(nullptr, c0, cnt, true);
+    for (int k = tid; k < cnt; k += QR_THREADS) {
+      orig[c0 + k] = est[c0 + k] = total(k).x;
+      again[c0 + k] = 0;
+    }
   }
   __syncthreads();
-  allreduce(coef, n, coef);
-  // sqrt is monotonic: the largest norm is the root of the largest square,
-  // taken once (FP64 square roots on every thread would load the narrow pipe)
-  if (threadIdx.x == 0) {
-    double m2 = 0.0;
-    for (int c = 0; c < n; ++c) m2 = fmax(m2, coef[c].x);
-    scal[4] = make_double2(sqrt(m2), 0.0);
-  }
-  __syncthreads();
-  const double tol = 1e-12 * scal[4].x;
+  // non-negative FP64 numbers order like their bit patterns
+  long long big = 0;
+  for (int c = 0; c < n; ++c) big = max(big, __double_as_longlong(orig[c]));
+
   int nq = 0;
-  for (int j = 0; j < n; ++j) {
-    for (int i = threadIdx.x; i < ml; i += blockDim.x) v[i] = A[(size_t)j * mc + i];
-    __syncthreads();
-    const int q = nq;
-    double nrm2;
-    if (q == 0) {
-      nrm2 = vnorm2();
-    } else {
-      // The first pass reduces the coefficients and |v|^2 together, and when
-      // it removed less than half of |v|^2 the residual norm follows from
-      // Pythagoras, |v'|^2 = |v|^2 - sum |c|^2 (accurate to a few ulp in that
-      // regime) -- one cluster reduction per column instead of three.
-      double before = 0.0;
-      nrm2 = 0.0;
-      for (int pass = 0; pass < 2; ++pass) {
-        if (pass == 0 && warp == nwarp - 1) {
-          double s2 = 0.0;
-          for (int i = lane; i < ml; i += 32) s2 += cabs2(v[i]);
-          s2 = warp_sum(s2);
-          if (lane == 0) coef[q] = make_double2(s2, 0.0);
-        }
-        for (int cc = warp; cc < q; cc += nwarp) {
-          const double2* qc = A + (size_t)cc * mc;
-          double re = 0.0, im = 0.0;
-          for (int i = lane; i < ml; i += 32) {
-            const double2 a = qc[i], b = v[i];
-            re += a.x * b.x + a.y * b.y;   // conj(q) * v
-            im += a.x * b.y - a.y * b.x;
+  for (int j = 0; j < n && nq < kmax; ++j) {
+    double2* v = A + (size_t)j * lda;
+    if (again[j]) {
+      // once more against the accepted columns
+      for (int c0 = 0; c0 < nq; c0 += NB) {
+        const int cnt = min(NB, nq - c0);
+        // conj(v) . q is the conjugate of q^H v
+        products(v, c0, cnt, false);
+        for (int k = tid; k < cnt; k += QR_THREADS) {
+          const double2 d = cconj(total(k));
+          fac[k] = cscale(d, 1.0 / piv[c0 + k]);
+          if (rank == 0) {
+            double2* rr = t.V + (size_t)j * n + c0 + k;
+            *rr = cadd(*rr, d);
           }
-          re = warp_sum(re);
-          im = warp_sum(im);
-          if (lane == 0) coef[cc] = make_double2(re, im);
         }
         __syncthreads();
-        allreduce(coef, pass == 0 ? q + 1 : q, coef);
-        if (pass == 0 && threadIdx.x == 0) {   // one thread; read after the barrier below
-          double proj = 0.0;
-          for (int cc = 0; cc < q; ++cc) proj += cabs2(coef[cc]);
-          scal[2] = make_double2(coef[q].x, proj);
-        }
-        for (int i = threadIdx.x; i < ml; i += blockDim.x) {
-          double2 acc = v[i];
-          for (int cc = 0; cc < q; ++cc) acc = csub(acc, cmul(coef[cc], A[(size_t)cc * mc + i]));
-          v[i] = acc;
-        }
-        if (rank == 0)
-          for (int cc = threadIdx.x; cc < q; cc += blockDim.x) {
-            double2* rr = t.V + (size_t)j * n + cc;   // R[cc, j], leading dimension n
-            *rr = cadd(*rr, coef[cc]);
+        // v -= sum_k q_k fac_k: `seg` threads per row, then their partial sums
+        const int seg = ml > 0 ? max(1, min(32, QR_THREADS / ml)) : 1;
+        const int rows = QR_THREADS / seg;
+        for (int i0 = 0; i0 < ml; i0 += rows) {
+          const int i = i0 + tid % rows, sg = tid / rows;
+          double2 acc = make_double2(0.0, 0.0);
+          if (i < ml && sg < seg)
+            for (int k = sg; k < cnt; k += seg) acc = cfma(fac[k], A[(size_t)(c0 + k) * lda + i], acc);
+          pp[tid] = acc;
+          __syncthreads();
+          if (tid < rows && i < ml) {
+            for (int s = 1; s < seg; ++s) acc = cadd(acc, pp[s * rows + tid]);
+            v[i] = csub(v[i], acc);
           }
-        __syncthreads();
-        if (pass == 0) {
-          before = scal[2].x;
-          const double est = before - scal[2].y;
-          if (!(est < 0.5 * before)) {   // one pass was enough
-            nrm2 = est;
-            break;
-          }
-        } else {
-          nrm2 = vnorm2();
+          __syncthreads();
         }
       }
     }
-    // the column norm and its inverse, once
-    if (threadIdx.x == 0) {
-      const double r0 = sqrt(nrm2);
-      scal[3] = make_double2(r0, r0 > 0.0 ? 1.0 / r0 : 0.0);
+    double inv = 0.0;
+    bool keep = false;
+    for (int c0 = j; c0 < n; c0 += NB) {
+      const int cnt = min(NB, n - c0);
+      products(v, c0, cnt, false);
+      // only the threads that form the factors of this batch touch the FP64 pipe
+      if (tid < cnt) {
+        bool ok = true;
+        if (c0 == j) {
+          const double pj = total(0).x;
+          ok = pj > 1e-24 * __longlong_as_double(big);
+          if (ok) inv = 1.0 / pj;
+          if (tid == 0) {
+            keep_sh = ok;
+            piv[nq] = pj;
+          }
+        }
+        for (int k = tid; ok && k < cnt; k += QR_THREADS) {
+          const double2 p = total(k);
+          const double2 f = cscale(p, inv);
+          fac[k] = f;
+          const double left = est[c0 + k] - (p.x * f.x + p.y * f.y);
+          est[c0 + k] = left;
+          again[c0 + k] = left < 0.5 * orig[c0 + k];
+          if (rank == 0) t.V[(size_t)(c0 + k) * n + nq] = p;   // scaled by 1 / |v| at the end
+        }
+      }
+      __syncthreads();
+      keep = keep_sh != 0;
+      if (!keep) break;
+      // a_c -= v f_c
+      const int k1 = c0 == j ? 1 : 0;
+      const int w = cnt - k1;
+      const int lpc = w * 8 <= QR_THREADS ? 8 : w * 4 <= QR_THREADS ? 4 : w * 2 <= QR_THREADS ? 2 : 1;
+      const int sub = tid & (lpc - 1);
+      for (int k = k1 + tid / lpc; k < cnt; k += QR_THREADS / lpc) {
+        const double2 f = make_double2(-fac[k].x, -fac[k].y);
+        double2* y = A + (size_t)(c0 + k) * lda;
+        for (int i = sub; i < ml; i += lpc) y[i] = cfma(f, v[i], y[i]);
+      }
+      __syncthreads();
     }
-    __syncthreads();
-    const double nrm = scal[3].x;
-    if (nrm > tol && q < kmax) {
-      const double inv = scal[3].y;
-      for (int i = threadIdx.x; i < ml; i += blockDim.x) A[(size_t)q * mc + i] = cscale(v[i], inv);
-      if (rank == 0 && threadIdx.x == 0) t.V[(size_t)j * n + q] = make_double2(nrm, 0.0);
-      nq = q + 1;
+    if (keep) {
+      if (nq != j) {
+        for (int i = tid; i < ml; i += QR_THREADS) A[(size_t)nq * lda + i] = v[i];
+        __syncthreads();
+      }
+      ++nq;
     }
-    __syncthreads();
   }
-  for (int c = 0; c < kmax; ++c)
-    for (int i = threadIdx.x; i < ml; i += blockDim.x)
-      t.A[(size_t)c * m + row0 + i] = c < nq ? A[(size_t)c * mc + i] : make_double2(0.0, 0.0);
+  __syncthreads();
+  // 1 / |v| of the accepted columns, once
+  for (int q = tid; q < nq; q += QR_THREADS) est[q] = 1.0 / sqrt(piv[q]);
+  __syncthreads();
+  for (int c = tid >> 5; c < kmax; c += QR_THREADS / 32)
+    for (int i = tid & 31; i < ml; i += 32)
+      t.A[(size_t)c * m + row0 + i] = c < nq ? cscale(A[c * lda + i], est[c]) : make_double2(0.0, 0.0);
+  if (rank == 0)
+    for (int e = tid; e < n * n; e += QR_THREADS) {
+      const int q = e % n;
+      if (q < nq) t.V[e] = cscale(t.V[e], est[q]);
+    }
   // no CTA may leave while others can still write into its slots
-  cl.sync();
+  if (CS > 1) cl.sync();
 }
 
 void launch_qr(const FactTask* d_tasks, int ntasks, cudaStream_t st, const FactTask* h_tasks) {
   if (ntasks <= 0) return;
-  // the cluster kernel pays off when some sector is large and all fit
-  size_t need = 0;
+  // A cluster per matrix when one of them is too much for one SM's FP64 pipe
+  // (4 m n^2 multiply-adds at 1.7 per clock), else a CTA per matrix, which
+  // saves the cluster barrier of every column.  The shared memory asked for
+  // is what the largest matrix needs; one that does not fit stays in global
+  // memory.
   bool large = false;
-  for (int i = 0; h_tasks && i < ntasks; ++i) {
-    need = std::max(need, qrc_elems(h_tasks[i].m, h_tasks[i].n) * sizeof(double2));
-    if (h_tasks[i].n >= 16 && (long long)h_tasks[i].m * h_tasks[i].n >= 2048) large = true;
+  for (int i = 0; i < ntasks; ++i)
+    if ((double)h_tasks[i].m * h_tasks[i].n * h_tasks[i].n >= QR_CLUSTER_WORK) large = true;
+  const int cs = large ? QR_CS : 1;
+  const size_t cap = QR_SMEM / sizeof(double2);
+  size_t need = 0;
+  bool fits = true;
+  for (int i = 0; i < ntasks; ++i) {
+    const int m = h_tasks[i].m, n = h_tasks[i].n;
+    const size_t e = qr_fixed(n, cs, QR_BATCH) + (size_t)qr_mc(m, cs) * n;
+    if (e > cap) fits = false;
+    need = std::max(need, std::min(e, cap));
   }
-  if (large && need <= (size_t)QR_SMEM) {
-    set_smem_limit((const void*)k_qr_cl, QR_SMEM);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(ntasks * QRC_CS));
-    cfg.blockDim = dim3(QRC_THREADS);
-    cfg.dynamicSmemBytes = need;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = QRC_CS;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, k_qr_cl, d_tasks);
+  const int batch = fits ? QR_BATCH : QR_BATCH_GLOBAL;
+  if (!fits) need = cap;
+  if (!large) {
+    set_smem_limit((const void*)k_qr<1>, QR_SMEM);
+    k_qr<1><<<ntasks, QR_THREADS, need * sizeof(double2), st>>>(d_tasks, batch, (int)need);
     return;
   }
-  set_smem_limit((const void*)k_qr, QR_SMEM);
-  k_qr<<<ntasks, QR_THREADS, QR_SMEM, st>>>(d_tasks);
+  set_smem_limit((const void*)k_qr<QR_CS>, QR_SMEM);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(ntasks * QR_CS));
+  cfg.blockDim = dim3(QR_THREADS);
+  cfg.dynamicSmemBytes = need * sizeof(double2);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = QR_CS;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k_qr<QR_CS>, d_tasks, batch, (int)need);
 }
-
 
 
 // ------------------------------------------------------------------ truncation rule
