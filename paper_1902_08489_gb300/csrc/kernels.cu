@@ -513,6 +513,295 @@ __global__ void __launch_bounds__(SVD_THREADS) k_svd(const FactTask* __restrict_
   }
 }
 
+// One-CTA Jacobi SVD of a small matrix (m x n, n <= m), in three stages:
+//   1. one-sided Jacobi in FP32 on a copy scaled by a power of two: this part's
+//      FP32 pipe is 64 times as wide as its FP64 pipe, so the sweeps that bring
+//      the columns from arbitrary to orthogonal within 1e-6 cost little;
+//   2. the accumulated rotations V, unitary to FP32 rounding, made unitary to
+//      FP64 rounding by two Newton steps V <- V - V (V^H V - 1) / 2 (the
+//      defect in FP64; the correction, a product of the small defect, in
+//      FP32), and A V in FP64;
+//   3. one-sided Jacobi in FP64 from there, to the same criterion as the
+//      kernels below.  Two or three sweeps remain of seven to nine.  A
+//      rotation's tangent is taken in FP32 (any tangent is a rotation; a
+//      relative error of 1e-7 in it leaves 1e-7 of the inner product), its
+//      cosine and sine in FP64, so V stays unitary to FP64 rounding.
+// What bounds it is the FP64 pipe in the rotations of stage 3 (12 operations
+// per row and pair of A and V).  Measured against FP64 Jacobi from the start
+// (one CTA below n = 24, a cluster from there): compression 256 -> 128 at L = 16
+// (15 launches, n <= 25) 17.3 -> 6.3 ms; a two-site Runge-Kutta step at L = 8,
+// D = 64 (224 launches, n <= 36) 76.4 -> 29.1 ms; at L = 12, D = 128 (n up to
+// 56) 342 -> 160 ms, of which 262 with the line at n = 32.  256 threads: 7.5 ms.
+constexpr int SVDS_THREADS = 512;
+constexpr int SVDS_MAX_N = 64;   // 164 KB of shared memory
+
+__host__ __device__ inline size_t svds_bytes(int m, int n) {
+  return 16 * ((size_t)m * n + (size_t)n * n) + 8 * (size_t)n * n;
+}
+
+__global__ void __launch_bounds__(SVDS_THREADS) k_svd_small(const FactTask* __restrict__ tasks,
+                                                            int* status) {
+  extern __shared__ double2 svd_sh[];
+  const FactTask t = tasks[blockIdx.x];
+  const int m = t.m, n = t.n;
+  double2* A = svd_sh;                        // [n][m], stage 3
+  double2* V = A + (size_t)m * n;             // [n][n]
+  float2* E = (float2*)(V + (size_t)n * n);   // [n][n], stage 2
+  float2* Af = (float2*)svd_sh;               // [n][m], stage 1, where A will be
+  float2* Vf = Af + (size_t)m * n;            // [n][n], stages 1 and 2, the same
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int NW = SVDS_THREADS / 32;
+  __shared__ int rotated, expo;
+  __shared__ double nrm[SVDS_MAX_N];          // squared column norms, tracked
+  __shared__ double2 pr[SVDS_MAX_N];          // per pair: c, whether it rotates
+  __shared__ double2 sc_sh[SVDS_MAX_N];       // per pair: s e^{i phi}
+  __shared__ int perm[SVDS_MAX_N];
+  if (tid == 0) expo = 0;
+  __syncthreads();
+  // power of two at the largest element, so that FP32 neither over- nor underflows
+  {
+    int e = 0;
+    for (int i = tid; i < m * n; i += SVDS_THREADS) {
+      const double2 x = t.A[i];
+      e = max(e, max((__double2hiint(x.x) >> 20) & 0x7ff, (__double2hiint(x.y) >> 20) & 0x7ff));
+    }
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (lane == 0) atomicMax(&expo, e);
+  }
+  __syncthreads();
+  const int ex = max(expo, 1) - 1022;         // |x| < 2^ex
+  const double down = scalbn(1.0, -max(-1000, min(1000, ex)));
+  for (int i = tid; i < m * n; i += SVDS_THREADS) {
+    const double2 x = t.A[i];
+    Af[i] = make_float2((float)(x.x * down), (float)(x.y * down));
+  }
+  for (int i = tid; i < n * n; i += SVDS_THREADS) Vf[i] = make_float2(i % n == i / n ? 1.f : 0.f, 0.f);
+  const int np = (n + 1) & ~1;   // even number of players
+  // the round's k-th pair, p < q; q == n: a bye
+  auto pair_of = [&](int k, int r, int& p, int& q) {
+    const int pb = np - 1 - k;
+    p = k == 0 ? 0 : ((k - 1 + r) % (np - 1)) + 1;
+    q = ((pb - 1 + r) % (np - 1)) + 1;
+    if (p > q) { const int x = p; p = q; q = x; }
+  };
+
+  // ---- stage 1: FP32, a warp per pair
+  for (int sweep = 0; sweep < 12 && expo < 0x7ff; ++sweep) {
+    __syncthreads();
+    if (tid == 0) rotated = 0;
+    __syncthreads();
+    for (int r = 0; r < np - 1; ++r) {
+      for (int k = warp; k < np / 2; k += NW) {
+        int p, q;
+        pair_of(k, r, p, q);
+        if (q >= n) continue;
+        float2 *ap = Af + (size_t)p * m, *aq = Af + (size_t)q * m;
+        float al = 0.f, be = 0.f, gr = 0.f, gi = 0.f;
+        for (int i = lane; i < m; i += 32) {
+          const float2 x = ap[i], y = aq[i];
+          al += x.x * x.x + x.y * x.y;
+          be += y.x * y.x + y.y * y.y;
+          gr += x.x * y.x + x.y * y.y;
+          gi += x.x * y.y - x.y * y.x;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          al += __shfl_xor_sync(0xffffffffu, al, o);
+          be += __shfl_xor_sync(0xffffffffu, be, o);
+          gr += __shfl_xor_sync(0xffffffffu, gr, o);
+          gi += __shfl_xor_sync(0xffffffffu, gi, o);
+        }
+        const float g2 = gr * gr + gi * gi;
+        if (!(al > 1e-30f && be > 1e-30f && g2 > 1e-12f * al * be && g2 > 1e-36f)) continue;
+        const float g = sqrtf(g2), z = (be - al) / (2.f * g);
+        const float tt = (z >= 0.f ? 1.f : -1.f) / (fabsf(z) + sqrtf(1.f + z * z));
+        const float c = 1.f / sqrtf(1.f + tt * tt);
+        const float sx = c * tt * gr / g, sy = c * tt * gi / g;
+        auto rot = [&](float2& x, float2& y) {
+          const float2 a = x, b = y;
+          x = make_float2(c * a.x - (sx * b.x + sy * b.y), c * a.y - (sx * b.y - sy * b.x));
+          y = make_float2(c * b.x + (sx * a.x - sy * a.y), c * b.y + (sx * a.y + sy * a.x));
+        };
+        for (int i = lane; i < m; i += 32) rot(ap[i], aq[i]);
+        for (int i = lane; i < n; i += 32) rot(Vf[(size_t)p * n + i], Vf[(size_t)q * n + i]);
+        if (lane == 0) rotated = 1;
+      }
+      __syncthreads();
+    }
+    if (!rotated) break;
+  }
+  __syncthreads();
+
+  // ---- stage 2: V unitary in FP64, then A V
+  for (int i = tid; i < n * n; i += SVDS_THREADS) V[i] = make_double2(Vf[i].x, Vf[i].y);
+  for (int it = 0; it < 2; ++it) {
+    __syncthreads();
+    for (int e = tid; e < n * n; e += SVDS_THREADS) {
+      const int p = e % n, q = e / n;
+      if (p > q) continue;
+      const double2 *x = V + (size_t)p * n, *y = V + (size_t)q * n;
+      double re = p == q ? -1.0 : 0.0, im = 0.0;
+      for (int i = 0; i < n; ++i) {
+        re = fma(x[i].x, y[i].x, fma(x[i].y, y[i].y, re));
+        im = fma(x[i].x, y[i].y, fma(-x[i].y, y[i].x, im));
+      }
+      const float2 d = make_float2((float)re, (float)im);
+      E[(size_t)q * n + p] = d;                     // (V^H V - 1)(p, q)
+      E[(size_t)p * n + q] = make_float2(d.x, p == q ? d.y : -d.y);
+    }
+    __syncthreads();
+    for (int e = tid; e < n * n; e += SVDS_THREADS) {
+      const int i = e % n, q = e / n;
+      float re = 0.f, im = 0.f;
+      for (int p = 0; p < n; ++p) {
+        const float2 v = Vf[(size_t)p * n + i], d = E[(size_t)q * n + p];
+        re += v.x * d.x - v.y * d.y;
+        im += v.x * d.y + v.y * d.x;
+      }
+      V[e] = make_double2(V[e].x - 0.5 * (double)re, V[e].y - 0.5 * (double)im);
+    }
+  }
+  __syncthreads();   // Vf is done with: A takes its place
+  for (int e = tid; e < m * n; e += SVDS_THREADS) {
+    const int i = e % m, q = e / m;
+    double2 acc = make_double2(0.0, 0.0);
+    for (int p = 0; p < n; ++p) acc = cfma(t.A[(size_t)p * m + i], V[(size_t)q * n + p], acc);
+    A[e] = cscale(acc, down);
+  }
+  __syncthreads();
+
+  // ---- stage 3: FP64
+  __shared__ double fro2;
+  // the computed inner product carries ~m eps relative rounding error
+  const double tol = 2.2e-16 * fmax(16.0, (double)m), tol2 = tol * tol;
+  int sweep = 0;
+  for (; sweep < SVD_MAX_SWEEPS; ++sweep) {
+    // column norms, four lanes each (tracked within the sweep)
+    for (int c = tid >> 2; c < ((n + 7) & ~7); c += SVDS_THREADS / 4) {
+      double s = 0.0;
+      if (c < n)
+        for (int i = tid & 3; i < m; i += 4) s += cabs2(A[(size_t)c * m + i]);
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      s += __shfl_xor_sync(0xffffffffu, s, 2);
+      if (c < n && (tid & 3) == 0) nrm[c] = s;
+    }
+    if (tid == 0) rotated = 0;
+    __syncthreads();
+    if (sweep == 0 && tid == 0) {
+      double f = 0.0;
+      for (int c = 0; c < n; ++c) f += nrm[c];
+      fro2 = f;
+    }
+    __syncthreads();
+    const double negl = 1e-26 * fro2;
+    for (int r = 0; r < np - 1; ++r) {
+      // inner products, four lanes per pair (whole warps enter: np / 2 * 4
+      // rounded up to 32)
+      for (int k0 = tid >> 2; k0 < ((np / 2 + 7) & ~7); k0 += SVDS_THREADS / 4) {
+        int p = 0, q = n;
+        if (k0 < np / 2) pair_of(k0, r, p, q);
+        double gr = 0.0, gi = 0.0;
+        if (q < n) {
+          const double2 *ap = A + (size_t)p * m, *aq = A + (size_t)q * m;
+          for (int i = tid & 3; i < m; i += 4) {
+            const double2 x = ap[i], y = aq[i];
+            gr = fma(x.x, y.x, fma(x.y, y.y, gr));
+            gi = fma(x.x, y.y, fma(-x.y, y.x, gi));
+          }
+        }
+        gr += __shfl_xor_sync(0xffffffffu, gr, 1);
+        gi += __shfl_xor_sync(0xffffffffu, gi, 1);
+        gr += __shfl_xor_sync(0xffffffffu, gr, 2);
+        gi += __shfl_xor_sync(0xffffffffu, gi, 2);
+        if ((tid & 3) == 0 && k0 < np / 2) {
+          double c = 1.0;
+          double2 s = make_double2(0.0, 0.0);
+          bool go = false;
+          if (q < n) {
+            const double al = nrm[p], be = nrm[q], g2 = gr * gr + gi * gi;
+            go = al > negl && be > negl && g2 > tol2 * al * be;
+            if (go) {
+              double tr, ti;   // tan e^{i phi}
+              if (g2 > 1e-32) {
+                const float gf = sqrtf((float)g2), z = (float)(be - al) / (2.f * gf);
+                const float tt = fabsf(z) > 1e9f ? 0.5f / z
+                                                 : copysignf(1.f, z) / (fabsf(z) + sqrtf(1.f + z * z));
+                tr = (double)(tt * ((float)gr / gf));
+                ti = (double)(tt * ((float)gi / gf));
+              } else {
+                const double g = sqrt(g2), z = (be - al) / (2.0 * g);
+                const double tt = (z >= 0.0 ? 1.0 : -1.0) / (fabs(z) + sqrt(1.0 + z * z));
+                tr = tt * gr / g;
+                ti = tt * gi / g;
+              }
+              const double h = tr * tr + ti * ti;
+              if (h < 1e-5)   // 1 / sqrt(1 + h), next term 63/256 h^5
+                c = 1.0 + h * (-0.5 + h * (0.375 + h * (-0.3125 + h * 0.2734375)));
+              else
+                c = 1.0 / sqrt(1.0 + h);
+              s = make_double2(c * tr, c * ti);
+              const double d = tr * gr + ti * gi;   // tan |g|
+              nrm[p] = al - d;
+              nrm[q] = be + d;
+              rotated = 1;
+            }
+          }
+          pr[k0] = make_double2(c, go ? 1.0 : 0.0);
+          sc_sh[k0] = s;
+        }
+      }
+      __syncthreads();
+      const int per = m + n;
+      for (int idx = tid; idx < (np / 2) * per; idx += SVDS_THREADS) {
+        const int k = idx / per, i = idx - k * per;
+        if (__double2hiint(pr[k].y) == 0) continue;
+        int p, q;
+        pair_of(k, r, p, q);
+        const double c = pr[k].x;
+        const double2 s = sc_sh[k];
+        double2* xp = i < m ? A + (size_t)p * m + i : V + (size_t)p * n + (i - m);
+        double2* yp = i < m ? A + (size_t)q * m + i : V + (size_t)q * n + (i - m);
+        const double2 x = *xp, y = *yp;
+        *xp = make_double2(fma(c, x.x, fma(-s.x, y.x, -s.y * y.y)), fma(c, x.y, fma(-s.x, y.y, s.y * y.x)));
+        *yp = make_double2(fma(c, y.x, fma(s.x, x.x, -s.y * x.y)), fma(c, y.y, fma(s.x, x.y, s.y * x.x)));
+      }
+      __syncthreads();
+    }
+    const int any = rotated;
+    __syncthreads();
+    if (!any) break;
+  }
+  if (tid == 0 && sweep == SVD_MAX_SWEEPS) atomicExch(status, 1);
+
+  // singular values, descending (ties: lower index first)
+  for (int c = warp; c < n; c += NW) {
+    double s = 0.0;
+    for (int i = lane; i < m; i += 32) s += cabs2(A[(size_t)c * m + i]);
+    s = warp_sum(s);
+    if (lane == 0) nrm[c] = sqrt(s);
+  }
+  if (tid < n) perm[tid] = tid;   // with NaN the ranks below do not cover every place
+  __syncthreads();
+  int rk = 0;
+  if (tid < n) {
+    const double sj = nrm[tid];
+    for (int k = 0; k < n; ++k) rk += (nrm[k] > sj) || (nrm[k] == sj && k < tid);
+    perm[rk] = tid;
+    pr[tid].x = sj > 0.0 ? 1.0 / sj : 0.0;
+  }
+  __syncthreads();
+  if (tid < n) t.s[tid] = nrm[perm[tid]] * scalbn(1.0, max(-1000, min(1000, ex)));
+  __syncthreads();
+  for (int e = tid; e < m * n; e += SVDS_THREADS) {
+    const int j = e / m, i = e % m, pj = perm[j];
+    t.A[e] = cscale(A[(size_t)pj * m + i], pr[pj].x);
+  }
+  for (int e = tid; e < n * n; e += SVDS_THREADS) {
+    const int j = e / n, i = e % n;
+    t.V[e] = V[(size_t)perm[j] * n + i];
+  }
+}
+
 // The same one-sided Jacobi SVD with one matrix spread over a cluster of
 // SVDC_CS CTAs: CTA `rank` holds rows [rank*mc, rank*mc + mc) of A in shared
 // memory and rows [rank*nc, rank*nc + nc) of V in global memory.  Each round
@@ -716,6 +1005,20 @@ __global__ void __launch_bounds__(SVDC_THREADS) k_svd_cl(const FactTask* __restr
 void launch_svd(const FactTask* d_tasks, int ntasks, int* d_status, cudaStream_t st,
                 size_t max_bytes, const FactTask* h_tasks) {
   if (ntasks <= 0) return;
+  {
+    size_t need = 0;
+    bool all_small = h_tasks != nullptr;
+    for (int i = 0; h_tasks && i < ntasks; ++i) {
+      if (h_tasks[i].n > SVDS_MAX_N || h_tasks[i].m < h_tasks[i].n) all_small = false;
+      need = std::max(need, svds_bytes(h_tasks[i].m, h_tasks[i].n));
+    }
+    const size_t cap_small = 200 * 1024;
+    if (all_small && need <= cap_small) {
+      set_smem_limit((const void*)k_svd_small, (int)cap_small);
+      k_svd_small<<<ntasks, SVDS_THREADS, need, st>>>(d_tasks, d_status);
+      return;
+    }
+  }
   {
     // the cluster kernel for square (or tall) matrices with a large one
     const size_t cap_cl = 200 * 1024;
