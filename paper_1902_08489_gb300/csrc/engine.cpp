@@ -92,7 +92,24 @@ void Inter::alloc(cudaStream_t st, bool zero) {
   if (zero) TD_CHECK_CUDA(cudaMemsetAsync(data->p, 0, size * esz(), st));
 }
 
+void Inter::build_lookup() const {
+  for (const auto& b : blocks) {
+    n_rg = std::max(n_rg, b.rg + 1);
+    n_g = std::max(n_g, b.g + 1);
+  }
+  lookup.assign((size_t)n_rg * 5 * n_g, -1);
+  for (int i = 0; i < (int)blocks.size(); ++i)
+    lookup[((size_t)blocks[i].rg * 5 + blocks[i].sig + 1) * n_g + blocks[i].g] = i;
+}
+
 // ------------------------------------------------------------------ context
+
+std::unique_ptr<GemmLists> Context::take_gemm_lists() {
+  if (gemm_lists.empty()) return std::make_unique<GemmLists>();
+  std::unique_ptr<GemmLists> l = std::move(gemm_lists.back());
+  gemm_lists.pop_back();
+  return l;
+}
 
 Context::Context(cudaStream_t s, int prec, size_t ring_bytes) : st(s), precision(prec) {
   seg_cap = ((ring_bytes / RING_SEGS) + 255) & ~(size_t)255;
@@ -124,16 +141,15 @@ Context::~Context() {
 }
 
 const void* Context::stage(const void* src, size_t bytes) {
-  size_t need = (bytes + 255) & ~(size_t)255;
+  std::memcpy(stage_room(bytes), src, bytes);
+  return stage_send(bytes);
+}
+
+char* Context::stage_room(size_t bytes) {
+  const size_t need = (bytes + 255) & ~(size_t)255;
   if (need > seg_cap) {
-    // oversize: dedicated buffer released after the stream passes it
-    DevPtr b = dev_alloc(need, st);
-    TD_CHECK_CUDA(cudaMemcpyAsync(b->p, src, bytes, cudaMemcpyHostToDevice, st));
-    wait_stream();
-    // its stream-ordered free is enqueued when the last holder lets go, so
-    // keeping it here until the context's next synchronisation is enough
-    oversize.push_back(b);
-    return b->p;
+    pack.resize(bytes);
+    return pack.data();
   }
   if (ring_off - (size_t)cur_seg * seg_cap + need > seg_cap) {
     // leave the current segment (all its consumers are enqueued by now)
@@ -144,7 +160,21 @@ const void* Context::stage(const void* src, size_t bytes) {
     cur_seg = next;
     ring_off = (size_t)next * seg_cap;
   }
-  std::memcpy(h_ring + ring_off, src, bytes);
+  return h_ring + ring_off;
+}
+
+const void* Context::stage_send(size_t bytes) {
+  const size_t need = (bytes + 255) & ~(size_t)255;
+  if (need > seg_cap) {
+    // oversize: dedicated buffer released after the stream passes it
+    DevPtr b = dev_alloc(need, st);
+    TD_CHECK_CUDA(cudaMemcpyAsync(b->p, pack.data(), bytes, cudaMemcpyHostToDevice, st));
+    wait_stream();
+    // its stream-ordered free is enqueued when the last holder lets go, so
+    // keeping it here until the context's next synchronisation is enough
+    oversize.push_back(b);
+    return b->p;
+  }
   TD_CHECK_CUDA(cudaMemcpyAsync(d_ring + ring_off, h_ring + ring_off, bytes,
                                 cudaMemcpyHostToDevice, st));
   const void* out = d_ring + ring_off;
@@ -276,6 +306,8 @@ void upload_mpo_tables(MPOd& m, Context& c) {
   m.tab_right_idx.assign(m.L, {});
   m.tab_left_flat.assign(m.L, {});
   m.tab_right_flat.assign(m.L, {});
+  m.nav_left.assign(m.L, {});
+  m.nav_right.assign(m.L, {});
   for (int i = 0; i < m.L; ++i) {
     const MPOBond& bi = m.bonds[i];
     const MPOBond& bo = m.bonds[i + 1];
@@ -332,6 +364,23 @@ void upload_mpo_tables(MPOd& m, Context& c) {
       m.tab_left_flat[i][(size_t)(kv.first[0] * 4 + kv.first[1]) * ngo + kv.first[2]] = kv.second;
     for (auto& kv : m.tab_right_idx[i])
       m.tab_right_flat[i][(size_t)(kv.first[0] * 4 + kv.first[1]) * ngi + kv.first[2]] = kv.second;
+    // charge of the output group: q_in + q_s - q_s' to the right, the reverse
+    // to the left
+    for (int dir = 0; dir < 2; ++dir) {
+      const MPOBond &bx = dir ? bo : bi, &by = dir ? bi : bo;
+      const std::vector<int>& flat = dir ? m.tab_right_flat[i] : m.tab_left_flat[i];
+      std::vector<MPOd::Nav>& nav = dir ? m.nav_right[i] : m.nav_left[i];
+      const int ngx = (int)bx.gq.size(), ngy = (int)by.gq.size();
+      nav.assign((size_t)ngx * 16, {-1, -1});
+      for (int gx = 0; gx < ngx; ++gx)
+        for (int sg = 0; sg < 4; ++sg)
+          for (int sp = 0; sp < 4; ++sp) {
+            const int g = by.find(dir ? bx.gq[gx] - SITE_Q[sg] + SITE_Q[sp]
+                                      : bx.gq[gx] + SITE_Q[sg] - SITE_Q[sp]);
+            const int tab = g < 0 ? -1 : flat[(size_t)(sg * 4 + sp) * ngy + g];
+            if (tab >= 0) nav[(size_t)(gx * 4 + sg) * 4 + sp] = {g, tab};
+          }
+    }
   }
   m.rowptr = dev_alloc(std::max<size_t>(rowptr.size(), 1) * sizeof(int), c.st);
   m.ent_w = dev_alloc(std::max<size_t>(ent_w.size(), 1) * sizeof(int), c.st);
@@ -363,13 +412,23 @@ namespace {
 struct GemmBatch {
   Context& c;
   bool fp64;
-  std::vector<GemmTask> tasks;
-  std::vector<GemmTerm> terms;
-  std::vector<GemmSeg> segs;
-  std::vector<SegOps> segops;
+  std::unique_ptr<GemmLists> lists;
+  std::vector<GemmTask>& tasks;
+  std::vector<GemmTerm>& terms;
+  std::vector<GemmSeg>& segs;
+  std::vector<SegOps>& segops;
   double flops = 0.0, bytes = 0.0;
   explicit GemmBatch(Context& ctx, bool force_fp64 = false)
-      : c(ctx), fp64(force_fp64 || ctx.precision == TDMPS_FP64) {}
+      : c(ctx), fp64(force_fp64 || ctx.precision == TDMPS_FP64), lists(ctx.take_gemm_lists()),
+        tasks(lists->tasks), terms(lists->terms), segs(lists->segs), segops(lists->segops) {
+    tasks.clear();
+    terms.clear();
+    segs.clear();
+    segops.clear();
+  }
+  ~GemmBatch() { c.gemm_lists.push_back(std::move(lists)); }
+  GemmBatch(const GemmBatch&) = delete;
+  GemmBatch& operator=(const GemmBatch&) = delete;
   // A task whose rows (dim 0) or columns (dim 1) are n output blocks of the
   // given sizes (GemmSeg); `other` is the extent of the other dimension.
   void task_seg(int dim, int n, void* const* Cs, const int* ldcs, const int* sizes, int other,
@@ -603,10 +662,11 @@ struct GemmBatch {
     auto tiles_n = [&](const GemmTask& t) {
       return fp64 ? f64_tiles_n(t.N, small, t.walk) : (t.N + bn - 1) / bn;
     };
-    std::vector<int> tile_task;
-    std::vector<GemmTask> tk;
+    std::vector<int>& tile_task = lists->tile_task;
+    std::vector<TcTile>& tc_tiles = lists->tiles;
+    tile_task.clear();
+    tc_tiles.clear();
     std::vector<int> split_ids;
-    std::vector<TcTile> tc_tiles;
     size_t part_elems = 0;
     // Split-K: long K runs are shared by several CTAs, each of which stores
     // its partial sum in a slice of a scratch buffer; a reduction adds the
@@ -617,7 +677,8 @@ struct GemmBatch {
     // per unit to amortise the partial-slice store and its reduction.
     const int kc = fp64 ? f64_stage_k() : tc_stage_k();
     const int per_sm = fp64 ? 4 : 3, min_chunks = fp64 ? 2 : 4;
-    std::vector<long long> stages(tasks.size(), 0);
+    std::vector<long long>& stages = lists->stages;
+    stages.assign(tasks.size(), 0);
     long long total = 0;
     for (size_t i = 0; i < tasks.size(); ++i) {
       GemmTask& t = tasks[i];
@@ -637,7 +698,7 @@ struct GemmBatch {
       t.splits = t.walk > 1 ? 1 : (int)std::min<long long>(64, std::max<long long>(1, stages[i] / chunk));
       t.part = nullptr;
       t.tile_base = (int)tile_task.size();
-      int id = (int)tk.size();
+      const int id = (int)i;
       if (!fp64) {
         // host-built tile descriptors: this task's K stages split evenly
         for (int sp = 0; sp < t.splits; ++sp) {
@@ -670,10 +731,9 @@ struct GemmBatch {
         t.part = (void*)(uintptr_t)part_elems;
         part_elems += (size_t)t.splits * t.M * t.N;
       }
-      tk.push_back(t);
-      for (int q = 0; q < t.tiles_m * tn * t.splits; ++q) tile_task.push_back(id);
+      if (fp64) tile_task.insert(tile_task.end(), (size_t)t.tiles_m * tn * t.splits, id);
     }
-    if (tile_task.empty()) return;
+    if (tile_task.empty() && tc_tiles.empty()) return;
     // the reduction of the split tasks in chunks of at most 512 elements (one
     // CTA of 256 threads each, two elements per thread): a few large tasks
     // still spread over every SM, with enough independent slice loads in
@@ -682,7 +742,7 @@ struct GemmBatch {
     constexpr int red_chunk = 512;
     std::vector<int> red;
     for (int id : split_ids) {
-      const int mn = tk[id].M * tk[id].N;
+      const int mn = tasks[id].M * tasks[id].N;
       for (int b = 0; b < mn; b += red_chunk) {
         red.push_back(id);
         red.push_back(b);
@@ -695,33 +755,31 @@ struct GemmBatch {
       // one buffer, slices addressed in units of the widest element type
       part = dev_alloc(part_elems * sizeof(double2), c.st);
       for (int id : split_ids) {
-        GemmTask& t = tk[id];
+        GemmTask& t = tasks[id];
         t.part = (char*)part->p + (size_t)(uintptr_t)t.part * sizeof(double2);
       }
     }
     // tasks, terms, the tile map and the split list go to the device in one
     // staged copy
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    const size_t o_terms = al(tk.size() * sizeof(GemmTask));
+    const size_t o_terms = al(tasks.size() * sizeof(GemmTask));
     const size_t o_split = o_terms + al(terms.size() * sizeof(GemmTerm));
     const size_t o_segs = o_split + al(red.size() * sizeof(int));
     const size_t o_segops = o_segs + al(segs.size() * sizeof(GemmSeg));
     const size_t o_tiles = o_segops + al(segops.size() * sizeof(SegOps));
     const size_t pk_bytes =
         o_tiles + (fp64 ? tile_task.size() * sizeof(int) : tc_tiles.size() * sizeof(TcTile));
-    std::vector<char>& pk = c.pack;
-    pk.resize(pk_bytes);
-    std::memcpy(pk.data(), tk.data(), tk.size() * sizeof(GemmTask));
-    if (!terms.empty()) std::memcpy(pk.data() + o_terms, terms.data(), terms.size() * sizeof(GemmTerm));
-    if (!red.empty()) std::memcpy(pk.data() + o_split, red.data(), red.size() * sizeof(int));
-    if (!segs.empty()) std::memcpy(pk.data() + o_segs, segs.data(), segs.size() * sizeof(GemmSeg));
-    if (!segops.empty())
-      std::memcpy(pk.data() + o_segops, segops.data(), segops.size() * sizeof(SegOps));
+    char* pk = c.stage_room(pk_bytes);
+    std::memcpy(pk, tasks.data(), tasks.size() * sizeof(GemmTask));
+    if (!terms.empty()) std::memcpy(pk + o_terms, terms.data(), terms.size() * sizeof(GemmTerm));
+    if (!red.empty()) std::memcpy(pk + o_split, red.data(), red.size() * sizeof(int));
+    if (!segs.empty()) std::memcpy(pk + o_segs, segs.data(), segs.size() * sizeof(GemmSeg));
+    if (!segops.empty()) std::memcpy(pk + o_segops, segops.data(), segops.size() * sizeof(SegOps));
     if (fp64)
-      std::memcpy(pk.data() + o_tiles, tile_task.data(), tile_task.size() * sizeof(int));
+      std::memcpy(pk + o_tiles, tile_task.data(), tile_task.size() * sizeof(int));
     else
-      std::memcpy(pk.data() + o_tiles, tc_tiles.data(), tc_tiles.size() * sizeof(TcTile));
-    const char* base = (const char*)c.stage(pk.data(), pk_bytes);
+      std::memcpy(pk + o_tiles, tc_tiles.data(), tc_tiles.size() * sizeof(TcTile));
+    const char* base = (const char*)c.stage_send(pk_bytes);
     const GemmTask* dt = (const GemmTask*)base;
     const GemmTerm* dm = terms.empty() ? nullptr : (const GemmTerm*)(base + o_terms);
     const int* dtt = (const int*)(base + o_tiles);
@@ -833,15 +891,9 @@ static Inter plan_lstage(Context& c, const Env& E, const SiteT& ket, const Bond&
                          int site = 0) {
   auto consumed = [&](const Inter::Blk& eb, int sp) {
     if (!m || m->identity) return bra_has(*bra, eb.rg, sp);
-    const MPOBond& bi = m->bonds[site];
-    const MPOBond& bo = m->bonds[site + 1];
-    const std::vector<int>& flat = m->tab_left_flat[site];
-    const int ngy = (int)bo.gq.size();
-    for (int s = 0; s < 4; ++s) {
-      if (!bra_has(*bra, eb.rg, s)) continue;
-      const int g = bo.find(bi.gq[eb.g] + SITE_Q[s] - SITE_Q[sp]);
-      if (g >= 0 && flat[(size_t)(s * 4 + sp) * ngy + g] >= 0) return true;
-    }
+    const MPOd::Nav* nav = &m->nav_left[site][(size_t)eb.g * 16 + sp];
+    for (int s = 0; s < 4; ++s)
+      if (nav[s * 4].tab >= 0 && bra_has(*bra, eb.rg, s)) return true;
     return false;
   };
   Inter X;
@@ -893,10 +945,7 @@ static Inter plan_wstage(Context& c, Inter&& X, const MPOd& m, int site, bool le
   if (wb.mpo && wb.mpo != &m) throw Error(TDMPS_ERR_INVALID_ARG, "mixed MPOs in one W batch");
   wb.mpo = &m;
   wb.et = X.et;
-  const MPOBond& bi = m.bonds[site];
-  const MPOBond& bo = m.bonds[site + 1];
-  const MPOBond& bx = left ? bi : bo;   // channels of the input
-  const MPOBond& by = left ? bo : bi;   // channels of the output
+  const MPOBond& by = m.bonds[left ? site + 1 : site];   // channels of the output
   // X blocks grouped by (row group, column sector), in that order; a flat
   // table replaces an ordered map (this runs for every launch)
   int nrg = 0, nk = 0;
@@ -907,11 +956,12 @@ static Inter plan_wstage(Context& c, Inter&& X, const MPOd& m, int site, bool le
   std::vector<std::array<int, 4>> groups((size_t)nrg * nk, std::array<int, 4>{-1, -1, -1, -1});
   for (int x = 0; x < (int)X.blocks.size(); ++x)
     groups[(size_t)X.blocks[x].rg * nk + X.blocks[x].k][X.blocks[x].sig] = x;
-  const std::vector<int>& flat = left ? m.tab_left_flat[site] : m.tab_right_flat[site];
-  const int ngy = (int)by.gq.size();
+  const std::vector<MPOd::Nav>& nav = left ? m.nav_left[site] : m.nav_right[site];
   Inter Y;
   struct P { int xs[4]; int tabs[4]; };
   std::vector<P> pend;
+  pend.reserve(X.blocks.size());
+  Y.blocks.reserve(X.blocks.size());
   for (size_t gi = 0; gi < groups.size(); ++gi) {
     const std::array<int, 4>& grp = groups[gi];
     if (grp[0] < 0 && grp[1] < 0 && grp[2] < 0 && grp[3] < 0) continue;
@@ -925,16 +975,11 @@ static Inter plan_wstage(Context& c, Inter&& X, const MPOd& m, int site, bool le
         p.tabs[sp] = -1;
         int x = grp[sp];
         if (x < 0) continue;
-        // charge of the output channel group
-        QN qy = left ? bx.gq[X.blocks[x].g] + SITE_Q[s] - SITE_Q[sp]
-                     : bx.gq[X.blocks[x].g] - SITE_Q[s] + SITE_Q[sp];
-        int g = by.find(qy);
-        if (g < 0) continue;
-        const int tab = flat[(size_t)(s * 4 + sp) * ngy + g];
-        if (tab < 0) continue;
-        gy = g;
+        const MPOd::Nav v = nav[(size_t)(X.blocks[x].g * 4 + s) * 4 + sp];
+        if (v.tab < 0) continue;
+        gy = v.g;
         p.xs[sp] = x;
-        p.tabs[sp] = tab;
+        p.tabs[sp] = v.tab;
         if (first < 0) first = x;
       }
       if (first < 0) continue;
@@ -944,6 +989,9 @@ static Inter plan_wstage(Context& c, Inter&& X, const MPOd& m, int site, bool le
   }
   Y.et = X.et;
   Y.alloc(c.st, false);
+  wb.tasks.reserve(wb.tasks.size() + Y.blocks.size());
+  const std::vector<WTable>& tabs = left ? m.tab_left[site] : m.tab_right[site];
+  const int rpi = wstage_rows_per_item();
   for (int y = 0; y < (int)Y.blocks.size(); ++y) {
     const Inter::Blk& yb = Y.blocks[y];
     WTask t{};
@@ -959,14 +1007,13 @@ static Inter plan_wstage(Context& c, Inter&& X, const MPOd& m, int site, bool le
       if (x < 0) { t.X[sp] = nullptr; t.win[sp] = 0; t.csr[sp] = -1; continue; }
       t.X[sp] = X.ptr(x);
       t.win[sp] = X.blocks[x].W;
-      const WTable& tb = (left ? m.tab_left[site] : m.tab_right[site])[pend[y].tabs[sp]];
+      const WTable& tb = tabs[pend[y].tabs[sp]];
       t.csr[sp] = tb.rowptr_off;
       nnz += tb.nnz;
       wb.bytes += (double)X.esz() * X.blocks[x].rows * X.blocks[x].W * X.blocks[x].cols;
     }
     int64_t n = (int64_t)yb.rows * yb.W * yb.cols;
     if (n >= ((int64_t)1 << 31)) throw Error(TDMPS_ERR_INVALID_ARG, "MPO-stage block too large");
-    const int rpi = wstage_rows_per_item();
     wb.work += (int64_t)((yb.rows + rpi - 1) / rpi) * yb.W * yb.cols;
     wb.bytes += (double)Y.esz() * n;
     // one real x complex multiply-add per non-zero W entry, row and column
@@ -1862,9 +1909,7 @@ MPSd fit(Context& c, const std::vector<FitTerm>& terms, const MPSd& guess, const
           E2[t].t.size = Y1[t].size;
           E2[t].t.et = Y1[t].et;
           for (auto& b : Y1[t].blocks) {
-            int id = (int)E2[t].t.blocks.size();
             E2[t].t.blocks.push_back({b.rg * 4 + b.sig, -1, b.g, b.k, b.rows, b.W, b.cols, b.off});
-            E2[t].t.index[Inter::key(b.rg * 4 + b.sig, -1, b.g, b.k)] = id;
           }
         }
         GemmBatch g2(c);

@@ -6,7 +6,6 @@
 #include <complex>
 #include <functional>
 #include <map>
-#include <unordered_map>
 #include <vector>
 
 #include "internal.hpp"
@@ -24,6 +23,18 @@ struct KStat {
 };
 
 struct Context;
+
+// The host arrays of one grouped GEMM launch; a context keeps the few it has
+// made, with their capacity, for the next launches.
+struct GemmLists {
+  std::vector<GemmTask> tasks;
+  std::vector<GemmTerm> terms;
+  std::vector<GemmSeg> segs;
+  std::vector<SegOps> segops;
+  std::vector<int> tile_task;
+  std::vector<TcTile> tiles;
+  std::vector<long long> stages;
+};
 
 // A worker of the instance batch: its own non-blocking stream and context
 // (staging ring, status words, MPO caches), used by one host thread at a time.
@@ -62,7 +73,9 @@ struct Context {
   struct Pending { int kind; cudaEvent_t a, b; };
   std::vector<Pending> pending;
   std::vector<cudaEvent_t> event_pool;   // recorded and read back events, reused
-  std::vector<char> pack;                // host packing buffer for staged task lists
+  std::vector<char> pack;                // host buffer of task lists larger than a ring segment
+  std::vector<std::unique_ptr<GemmLists>> gemm_lists;   // free GEMM lists (engine.cpp)
+  std::unique_ptr<GemmLists> take_gemm_lists();
   // scratch for device status words
   DevPtr status;   // int[16]: [0] SVD convergence, [4..5] Krylov, [8] tensor-core waits
   std::unique_ptr<MPOd> ident;   // identity MPO cache (by L)
@@ -78,6 +91,10 @@ struct Context {
 
   // copy a host array into device memory valid until the stream passes it
   const void* stage(const void* src, size_t bytes);
+  // the same in two steps: room for `bytes` (host memory to fill, before any
+  // other staging call), then the copy, which returns the device address
+  char* stage_room(size_t bytes);
+  const void* stage_send(size_t bytes);
   template <class T> const T* stage(const std::vector<T>& v) {
     return v.empty() ? nullptr : (const T*)stage(v.data(), v.size() * sizeof(T));
   }
@@ -104,7 +121,8 @@ struct Context {
 // ------------------------------------------------------------------ intermediates
 
 // Block-sparse tensor with blocks rows x W x cols keyed (row group, sigma,
-// channel group, column sector); sigma = -1 for environments.
+// channel group, column sector); sigma = -1 for environments.  Blocks are
+// added before the first find().
 struct Inter {
   struct Blk {
     int rg, sig, g, k;
@@ -112,29 +130,31 @@ struct Inter {
     size_t off;
   };
   std::vector<Blk> blocks;
-  std::unordered_map<uint64_t, int> index;   // key(rg, sig, g, k) -> block id
   size_t size = 0;
   int et = 0;   // element type: 0 complex double, 1 complex float
   DevPtr data;
   size_t esz() const { return et ? sizeof(float2) : sizeof(double2); }
-  // sector, channel-group and local-state indices are small: 16 bits each
-  static uint64_t key(int rg, int sig, int g, int k) {
-    return ((uint64_t)(uint16_t)rg << 48) | ((uint64_t)(uint16_t)(sig + 1) << 32) |
-           ((uint64_t)(uint16_t)g << 16) | (uint64_t)(uint16_t)k;
-  }
+  // block (rg, sig, g) with column sector k (charge conservation leaves one k
+  // per (rg, sig, g)), or -1.  The lookup table is made on first use: most
+  // intermediates are only walked.
   int find(int rg, int sig, int g, int k) const {
-    auto it = index.find(key(rg, sig, g, k));
-    return it == index.end() ? -1 : it->second;
+    if (lookup.empty() && !blocks.empty()) build_lookup();
+    if (rg >= n_rg || g >= n_g) return -1;
+    const int id = lookup[((size_t)rg * 5 + sig + 1) * n_g + g];
+    return id >= 0 && blocks[id].k == k ? id : -1;
   }
   int add(int rg, int sig, int g, int k, int rows, int W, int cols) {
-    int id = (int)blocks.size();
     blocks.push_back({rg, sig, g, k, rows, W, cols, size});
-    index[key(rg, sig, g, k)] = id;
     size += (size_t)rows * W * cols;
-    return id;
+    return (int)blocks.size() - 1;
   }
   void* ptr(int b) const { return (char*)data->p + blocks[b].off * esz(); }
   void alloc(cudaStream_t st, bool zero);
+
+ private:
+  mutable std::vector<int> lookup;   // [(rg * 5 + sig + 1) * n_g + g]
+  mutable int n_rg = 0, n_g = 0;
+  void build_lookup() const;
 };
 
 // Environment E[a, w, a'] at one bond: rows = bra row groups, channels = MPO

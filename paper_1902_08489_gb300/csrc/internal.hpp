@@ -155,6 +155,10 @@ struct MPOd {
   std::vector<std::map<std::array<int, 3>, int>> tab_left_idx, tab_right_idx;
   // the same lookups as flat arrays: [(sig*4 + sigp) * ngroups + g] -> table or -1
   std::vector<std::vector<int>> tab_left_flat, tab_right_flat;
+  // per site, [(g_in * 4 + sig) * 4 + sigp] over the channel groups g_in of the
+  // stage's input: output group and table, -1 where there is none
+  struct Nav { int g, tab; };
+  std::vector<std::vector<Nav>> nav_left, nav_right;
   DevPtr rowptr, ent_w, ent_v, ent_vf;        // int, int, double, float
   int64_t n_elem = 0;
 };
