@@ -1372,7 +1372,8 @@ struct FactWork {
   std::vector<size_t> a_off, v_off, s_off;
 };
 
-// allocate m x n work matrices (+ n x n V / R, + n values) for a list of shapes
+// allocate m x n work matrices (+ n x n V / R, + n values, those of all shapes
+// side by side at the end) for a list of shapes
 FactWork fact_alloc(Context& c, const std::vector<std::pair<int, int>>& shapes) {
   FactWork fw;
   size_t off = 0;
@@ -1383,9 +1384,10 @@ FactWork fact_alloc(Context& c, const std::vector<std::pair<int, int>>& shapes) 
     fw.v_off.push_back(off);
     off += (size_t)sh.second * sh.second * sizeof(double2);
     off = (off + 255) & ~(size_t)255;
+  }
+  for (auto& sh : shapes) {
     fw.s_off.push_back(off);
     off += (size_t)sh.second * sizeof(double);
-    off = (off + 255) & ~(size_t)255;
   }
   fw.buf = dev_alloc(std::max<size_t>(off, 256), c.st);
   char* base = (char*)fw.buf->p;
@@ -1645,8 +1647,7 @@ static SplitResult svd_split(Context& c, const SiteT& Th, const RowGroups& rows,
       }
   }
   // zero the work matrices first (blocks not present stay zero)
-  for (size_t i = 0; i < qs.size(); ++i)
-    launch_zero(fw.tasks[i].A, (size_t)shapes[i].first * shapes[i].second, c.st);
+  TD_CHECK_CUDA(cudaMemsetAsync(fw.buf->p, 0, fw.buf->bytes, c.st));
   run_copy(c, g, 1);
   // QR-preconditioned one-sided Jacobi: M = Q R, Jacobi on W = R^H gives
   // W J = U_w S, hence M = (Q J) S U_w^H; far fewer sweeps than Jacobi on M
@@ -1684,12 +1685,10 @@ static SplitResult svd_split(Context& c, const SiteT& Th, const RowGroups& rows,
   int nv = 0;
   int ntot = 0;
   for (auto& sh : shapes) ntot += sh.second;
-  DevPtr svals = dev_alloc(sizeof(double) * std::max(1, ntot) * 2 + 64, c.st);
+  DevPtr svals = dev_alloc(sizeof(double) * std::max(1, ntot) + 64, c.st);   // sorted
   DevPtr sids = dev_alloc(sizeof(int) * std::max(1, ntot) * 2 + 64, c.st);
   for (size_t i = 0; i < qs.size(); ++i) {
-    TD_CHECK_CUDA(cudaMemcpyAsync((double*)svals->p + nv, fj.tasks[i].s,
-                                  sizeof(double) * shapes[i].second, cudaMemcpyDeviceToDevice, c.st));
-    for (int k = 0; k < shapes[i].second; ++k) secid.push_back((int)i);
+    secid.insert(secid.end(), shapes[i].second, (int)i);
     nv += shapes[i].second;
   }
   const int* dsec = c.stage(secid);
@@ -1699,8 +1698,9 @@ static SplitResult svd_split(Context& c, const SiteT& Th, const RowGroups& rows,
   {
     cudaEvent_t ev;
     c.kbegin(TDMPS_KSTAT_OTHER, &ev);
-    launch_trunc((const double*)svals->p, dsec, nv, (int)qs.size(), D, eps, dkept, dw,
-                 (double*)svals->p + ntot, (int*)sids->p, c.st);
+    // the values of all sectors lie side by side (fact_alloc)
+    launch_trunc(fj.tasks[0].s, dsec, nv, (int)qs.size(), D, eps, dkept, dw, (double*)svals->p,
+                 (int*)sids->p, c.st);
     c.kend(TDMPS_KSTAT_OTHER, ev, 0.0, 0.0);
   }
   std::vector<int> hk(qs.size());
