@@ -298,72 +298,99 @@ const MPOd& Context::rdm_mpo(int L) {
 // ------------------------------------------------------------------ MPO tables
 
 void upload_mpo_tables(MPOd& m, Context& c) {
-  std::vector<int> rowptr, ent_w;
+  std::vector<int> rowptr, ent_w, grp_ptr, grp_w;
   std::vector<double> ent_v;
+  std::vector<float> grp_v;
   m.tab_left.assign(m.L, {});
   m.tab_right.assign(m.L, {});
-  m.tab_left_idx.assign(m.L, {});
-  m.tab_right_idx.assign(m.L, {});
   m.tab_left_flat.assign(m.L, {});
   m.tab_right_flat.assign(m.L, {});
   m.nav_left.assign(m.L, {});
   m.nav_right.assign(m.L, {});
+  const int G = wstage_group();
+  std::vector<int> start, order, slot, cols;
   for (int i = 0; i < m.L; ++i) {
     const MPOBond& bi = m.bonds[i];
     const MPOBond& bo = m.bonds[i + 1];
-    // left: key (sig, sigp, g_out) rows over w_out
-    std::map<std::array<int, 3>, std::vector<const WElem*>> L, R;
-    for (const WElem& e : m.W[i]) {
-      L[{e.sig, e.sigp, bo.ch_group[e.wout]}].push_back(&e);
-      R[{e.sig, e.sigp, bi.ch_group[e.win]}].push_back(&e);
+    // left: tables (sig, sigp, g_out) with rows over w_out; right: (sig, sigp,
+    // g_in) with rows over w_in
+    for (int dir = 0; dir < 2; ++dir) {
+      const MPOBond &bx = dir ? bo : bi, &by = dir ? bi : bo;   // columns, rows of the tables
+      const int ngy = (int)by.gq.size(), nch = by.nch();
+      std::vector<int>& flat = dir ? m.tab_right_flat[i] : m.tab_left_flat[i];
+      std::vector<WTable>& tabs = dir ? m.tab_right[i] : m.tab_left[i];
+      flat.assign((size_t)16 * ngy, -1);
+      auto row_of = [&](const WElem& e) { return dir ? e.win : e.wout; };
+      auto col_of = [&](const WElem& e) { return dir ? e.wout : e.win; };
+      // elements by (sig, sigp, row channel), each in the order of W (counting sort)
+      start.assign((size_t)16 * nch + 1, 0);
+      for (const WElem& e : m.W[i]) start[(size_t)(e.sig * 4 + e.sigp) * nch + row_of(e) + 1]++;
+      for (size_t k = 1; k < start.size(); ++k) start[k] += start[k - 1];
+      order.resize(m.W[i].size());
+      slot.assign(start.begin(), start.end() - 1);
+      for (int k = 0; k < (int)m.W[i].size(); ++k) {
+        const WElem& e = m.W[i][k];
+        order[slot[(size_t)(e.sig * 4 + e.sigp) * nch + row_of(e)]++] = k;
+      }
+      // channels of each row group, by their place in it
+      std::vector<std::vector<int>> chan(ngy);
+      for (int gy = 0; gy < ngy; ++gy) chan[gy].resize(by.gsize[gy]);
+      for (int ch = 0; ch < nch; ++ch) chan[by.ch_group[ch]][by.ch_local[ch]] = ch;
+      slot.assign(bx.nch(), -1);   // column -> entry of the current channel group
+      for (int ss = 0; ss < 16; ++ss)
+        for (int gy = 0; gy < ngy; ++gy) {
+          const int rows = by.gsize[gy];
+          int gx = -1, nnz = 0;
+          for (int r = 0; r < rows; ++r) {
+            const size_t key = (size_t)ss * nch + chan[gy][r];
+            for (int q = start[key]; q < start[key + 1]; ++q) {
+              const int g = bx.ch_group[col_of(m.W[i][order[q]])];
+              if (gx >= 0 && g != gx) throw Error(TDMPS_ERR_SECTOR, "MPO charge inconsistency");
+              gx = g;
+              ++nnz;
+            }
+          }
+          if (!nnz) continue;
+          flat[(size_t)ss * ngy + gy] = (int)tabs.size();
+          WTable t{ss / 4, ss % 4, dir ? gx : gy, dir ? gy : gx, rows, (int)rowptr.size(), nnz,
+                   (int)grp_ptr.size()};
+          for (int r0 = 0; r0 < rows; r0 += G) {
+            grp_ptr.push_back((int)grp_w.size());
+            cols.clear();
+            for (int r = r0; r < std::min(rows, r0 + G); ++r) {
+              rowptr.push_back((int)ent_w.size());
+              const size_t key = (size_t)ss * nch + chan[gy][r];
+              for (int q = start[key]; q < start[key + 1]; ++q) {
+                const WElem& e = m.W[i][order[q]];
+                const int x = bx.ch_local[col_of(e)];
+                ent_w.push_back(x);
+                ent_v.push_back(e.v);
+                if (slot[x] < 0) {
+                  slot[x] = 0;
+                  cols.push_back(x);
+                }
+              }
+            }
+            // the input channels of the group, ascending, with a value per row
+            std::sort(cols.begin(), cols.end());
+            const size_t first = grp_w.size();
+            for (size_t k = 0; k < cols.size(); ++k) slot[cols[k]] = (int)(first + k);
+            grp_w.insert(grp_w.end(), cols.begin(), cols.end());
+            grp_v.resize(grp_w.size() * G, 0.f);
+            for (int r = r0; r < std::min(rows, r0 + G); ++r) {
+              const size_t key = (size_t)ss * nch + chan[gy][r];
+              for (int q = start[key]; q < start[key + 1]; ++q) {
+                const WElem& e = m.W[i][order[q]];
+                grp_v[(size_t)slot[bx.ch_local[col_of(e)]] * G + (r - r0)] += (float)e.v;
+              }
+            }
+            for (int x : cols) slot[x] = -1;
+          }
+          rowptr.push_back((int)ent_w.size());
+          grp_ptr.push_back((int)grp_w.size());
+          tabs.push_back(t);
+        }
     }
-    for (auto& kv : L) {
-      int gout = kv.first[2];
-      int rows = bo.gsize[gout];
-      int gin = bi.ch_group[kv.second[0]->win];
-      std::vector<std::vector<std::pair<int, double>>> perrow(rows);
-      for (auto* e : kv.second) {
-        if (bi.ch_group[e->win] != gin) throw Error(TDMPS_ERR_SECTOR, "MPO charge inconsistency");
-        perrow[bo.ch_local[e->wout]].push_back({bi.ch_local[e->win], e->v});
-      }
-      WTable t{kv.first[0], kv.first[1], gout, gin, rows, (int)rowptr.size(), 0};
-      const int first = (int)ent_w.size();
-      for (int r = 0; r < rows; ++r) {
-        rowptr.push_back((int)ent_w.size());
-        for (auto& pv : perrow[r]) { ent_w.push_back(pv.first); ent_v.push_back(pv.second); }
-      }
-      rowptr.push_back((int)ent_w.size());
-      t.nnz = (int)ent_w.size() - first;
-      m.tab_left_idx[i][kv.first] = (int)m.tab_left[i].size();
-      m.tab_left[i].push_back(t);
-    }
-    for (auto& kv : R) {
-      int gin = kv.first[2];
-      int rows = bi.gsize[gin];
-      int gout = bo.ch_group[kv.second[0]->wout];
-      std::vector<std::vector<std::pair<int, double>>> perrow(rows);
-      for (auto* e : kv.second) {
-        if (bo.ch_group[e->wout] != gout) throw Error(TDMPS_ERR_SECTOR, "MPO charge inconsistency");
-        perrow[bi.ch_local[e->win]].push_back({bo.ch_local[e->wout], e->v});
-      }
-      WTable t{kv.first[0], kv.first[1], gout, gin, rows, (int)rowptr.size(), 0};
-      const int first = (int)ent_w.size();
-      for (int r = 0; r < rows; ++r) {
-        rowptr.push_back((int)ent_w.size());
-        for (auto& pv : perrow[r]) { ent_w.push_back(pv.first); ent_v.push_back(pv.second); }
-      }
-      rowptr.push_back((int)ent_w.size());
-      t.nnz = (int)ent_w.size() - first;
-      m.tab_right_idx[i][kv.first] = (int)m.tab_right[i].size();
-      m.tab_right[i].push_back(t);
-    }
-    const int ngo = (int)bo.gq.size(), ngi = (int)bi.gq.size();
-    m.tab_left_flat[i].assign((size_t)16 * ngo, -1);
-    m.tab_right_flat[i].assign((size_t)16 * ngi, -1);
-    for (auto& kv : m.tab_left_idx[i])
-      m.tab_left_flat[i][(size_t)(kv.first[0] * 4 + kv.first[1]) * ngo + kv.first[2]] = kv.second;
-    for (auto& kv : m.tab_right_idx[i])
-      m.tab_right_flat[i][(size_t)(kv.first[0] * 4 + kv.first[1]) * ngi + kv.first[2]] = kv.second;
     // charge of the output group: q_in + q_s - q_s' to the right, the reverse
     // to the left
     for (int dir = 0; dir < 2; ++dir) {
@@ -382,22 +409,17 @@ void upload_mpo_tables(MPOd& m, Context& c) {
           }
     }
   }
-  m.rowptr = dev_alloc(std::max<size_t>(rowptr.size(), 1) * sizeof(int), c.st);
-  m.ent_w = dev_alloc(std::max<size_t>(ent_w.size(), 1) * sizeof(int), c.st);
-  m.ent_v = dev_alloc(std::max<size_t>(ent_v.size(), 1) * sizeof(double), c.st);
-  m.ent_vf = dev_alloc(std::max<size_t>(ent_v.size(), 1) * sizeof(float), c.st);
-  std::vector<float> ent_vf(ent_v.begin(), ent_v.end());
-  if (!rowptr.empty())
-    TD_CHECK_CUDA(cudaMemcpyAsync(m.rowptr->p, rowptr.data(), rowptr.size() * sizeof(int),
-                                  cudaMemcpyHostToDevice, c.st));
-  if (!ent_w.empty()) {
-    TD_CHECK_CUDA(cudaMemcpyAsync(m.ent_w->p, ent_w.data(), ent_w.size() * sizeof(int),
-                                  cudaMemcpyHostToDevice, c.st));
-    TD_CHECK_CUDA(cudaMemcpyAsync(m.ent_v->p, ent_v.data(), ent_v.size() * sizeof(double),
-                                  cudaMemcpyHostToDevice, c.st));
-    TD_CHECK_CUDA(cudaMemcpyAsync(m.ent_vf->p, ent_vf.data(), ent_vf.size() * sizeof(float),
-                                  cudaMemcpyHostToDevice, c.st));
-  }
+  auto send = [&](const void* src, size_t bytes) {
+    DevPtr d = dev_alloc(std::max<size_t>(bytes, 16), c.st);
+    if (bytes) TD_CHECK_CUDA(cudaMemcpyAsync(d->p, src, bytes, cudaMemcpyHostToDevice, c.st));
+    return d;
+  };
+  m.rowptr = send(rowptr.data(), rowptr.size() * sizeof(int));
+  m.ent_w = send(ent_w.data(), ent_w.size() * sizeof(int));
+  m.ent_v = send(ent_v.data(), ent_v.size() * sizeof(double));
+  m.grp_ptr = send(grp_ptr.data(), grp_ptr.size() * sizeof(int));
+  m.grp_w = send(grp_w.data(), grp_w.size() * sizeof(int));
+  m.grp_v = send(grp_v.data(), grp_v.size() * sizeof(float));
   // host vectors must outlive the async copies
   c.wait_stream();
 }
@@ -814,8 +836,9 @@ struct WBatch {
     const WTask* dt = c.stage(tasks);
     cudaEvent_t ev;
     c.kbegin(TDMPS_KSTAT_WSTAGE, &ev);
-    launch_wstage(dt, (int)tasks.size(), work, (const int*)m.rowptr->p, (const int*)m.ent_w->p,
-                  (const double*)m.ent_v->p, (const float*)m.ent_vf->p, et, c.st);
+    const WTables tb{(const int*)m.rowptr->p, (const int*)m.ent_w->p, (const double*)m.ent_v->p,
+                     (const int*)m.grp_ptr->p, (const int*)m.grp_w->p, (const float*)m.grp_v->p};
+    launch_wstage(dt, (int)tasks.size(), work, tb, et, c.st);
     c.kend(TDMPS_KSTAT_WSTAGE, ev, flops, bytes);
   }
 };
@@ -991,7 +1014,6 @@ static Inter plan_wstage(Context& c, Inter&& X, const MPOd& m, int site, bool le
   Y.alloc(c.st, false);
   wb.tasks.reserve(wb.tasks.size() + Y.blocks.size());
   const std::vector<WTable>& tabs = left ? m.tab_left[site] : m.tab_right[site];
-  const int rpi = wstage_rows_per_item();
   for (int y = 0; y < (int)Y.blocks.size(); ++y) {
     const Inter::Blk& yb = Y.blocks[y];
     WTask t{};
@@ -1008,13 +1030,13 @@ static Inter plan_wstage(Context& c, Inter&& X, const MPOd& m, int site, bool le
       t.X[sp] = X.ptr(x);
       t.win[sp] = X.blocks[x].W;
       const WTable& tb = tabs[pend[y].tabs[sp]];
-      t.csr[sp] = tb.rowptr_off;
+      t.csr[sp] = X.et ? tb.grp_off : tb.rowptr_off;
       nnz += tb.nnz;
       wb.bytes += (double)X.esz() * X.blocks[x].rows * X.blocks[x].W * X.blocks[x].cols;
     }
     int64_t n = (int64_t)yb.rows * yb.W * yb.cols;
     if (n >= ((int64_t)1 << 31)) throw Error(TDMPS_ERR_INVALID_ARG, "MPO-stage block too large");
-    wb.work += (int64_t)((yb.rows + rpi - 1) / rpi) * yb.W * yb.cols;
+    wb.work += wstage_items(yb.rows, yb.W, yb.cols, X.et);
     wb.bytes += (double)Y.esz() * n;
     // one real x complex multiply-add per non-zero W entry, row and column
     wb.flops += 4.0 * (double)nnz * yb.rows * yb.cols;

@@ -143,6 +143,7 @@ struct WTable {
   int rows;         // rows of the CSR (W_gout for left, W_gin for right)
   int rowptr_off;   // offset into rowptr array
   int nnz;          // non-zero entries of the table
+  int grp_off;      // offset into grp_ptr (groups of output channels, FP32)
 };
 
 struct MPOd {
@@ -152,14 +153,14 @@ struct MPOd {
   std::vector<std::vector<WElem>> W;          // per site
   // device tables
   std::vector<std::vector<WTable>> tab_left, tab_right;
-  std::vector<std::map<std::array<int, 3>, int>> tab_left_idx, tab_right_idx;
-  // the same lookups as flat arrays: [(sig*4 + sigp) * ngroups + g] -> table or -1
+  // [(sig*4 + sigp) * ngroups + g] -> table or -1
   std::vector<std::vector<int>> tab_left_flat, tab_right_flat;
   // per site, [(g_in * 4 + sig) * 4 + sigp] over the channel groups g_in of the
   // stage's input: output group and table, -1 where there is none
   struct Nav { int g, tab; };
   std::vector<std::vector<Nav>> nav_left, nav_right;
-  DevPtr rowptr, ent_w, ent_v, ent_vf;        // int, int, double, float
+  DevPtr rowptr, ent_w, ent_v;                // int, int, double
+  DevPtr grp_ptr, grp_w, grp_v;               // int, int, float x wstage_group()
   int64_t n_elem = 0;
 };
 

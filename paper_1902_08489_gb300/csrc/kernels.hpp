@@ -73,7 +73,7 @@ struct WTask {
   void* Y;
   const void* X[4];
   int win[4];
-  int csr[4];          // row-pointer offset of the CSR for input s (-1: none)
+  int csr[4];          // offset of input s's table in rowptr (FP64) or grp_ptr (FP32); -1: none
   int rows, wout, cols, beta;
   int64_t work_base;   // first flat element index of this task
 };
@@ -119,13 +119,19 @@ int f64_stage_k();                  // complex K per step; split-K shares out wh
 void launch_gemm(const GemmTask* d_tasks, const GemmTerm* d_terms, const GemmSeg* d_segs,
                  const SegOps* d_segops, const int* d_tile_task, int ntiles, bool small,
                  cudaStream_t st);
-// et: element type of X and Y (0 double2 with the FP64 values, 1 float2 with
-// the FP32 copy of the values)
-// rows a of a W-stage block that one work item covers (work per block:
-// ceil(rows / this) x wout x cols)
-int wstage_rows_per_item();
-void launch_wstage(const WTask* d_tasks, int ntasks, int64_t total_work, const int* d_rowptr,
-                   const int* d_ent_w, const double* d_ent_v, const float* d_ent_vf, int et,
+// Device tables of the MPO stage: CSR rows of single output channels (complex
+// FP64 data), and groups of wstage_group() consecutive output channels, each
+// a list of input channels with one value per output channel (complex FP32).
+struct WTables {
+  const int *rowptr, *ent_w;
+  const double* ent_v;
+  const int *grp_ptr, *grp_w;
+  const float* grp_v;   // wstage_group() per entry, 16-byte aligned
+};
+// et: element type of X and Y (0 double2, 1 float2)
+int64_t wstage_items(int rows, int wout, int cols, int et);   // work items of one output block
+int wstage_group();
+void launch_wstage(const WTask* d_tasks, int ntasks, int64_t total_work, const WTables& tb, int et,
                    cudaStream_t st);
 // One tile of the tensor-core GEMM, built on the host: rows m0.. (tc_tile_m()
 // of them), complex columns n0 .. n0 + ncols (ncols <= tc_tile_n()), and the
