@@ -146,7 +146,7 @@ struct TcTile {
 };
 // tensor-core grouped GEMM (kernels_tc.cu); mode 0 TF32, 1 3xTF32, 2 BF16;
 // operands complex float, C complex double (tc = 0) or float (tc = 1);
-// persistent: min(ntiles, n_sm) CTAs walk the tile list
+// persistent: min(ntiles, 2 n_sm) CTAs walk the tile list
 void launch_gemm_tc(const GemmTask* d_tasks, const GemmTerm* d_terms, const TcTile* d_tiles,
                     const GemmSeg* d_segs, const SegOps* d_segops, int ntiles, int mode, int n_sm,
                     int* d_err, cudaStream_t st);

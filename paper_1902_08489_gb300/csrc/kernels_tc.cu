@@ -13,7 +13,7 @@
 // TF32 tail and accumulates hi*hi + hi*lo + lo*hi; BF16 rounds both operands
 // to BF16 (kind::f16, FP32 accumulation).
 //
-// The kernel is persistent (one CTA per SM walking a host-built tile list)
+// The kernel is persistent (two CTAs per SM walking a host-built tile list)
 // and warp-specialised:
 //   warps 0..7   producers.  The symmetry blocks are ragged and addressed
 //                through arbitrary leading dimensions and operand modes, so
@@ -57,8 +57,17 @@ constexpr int TC_KR = 2 * TC_BKC; // real K per stage (16 tf32 = 2 MMA k-steps)
 constexpr int TC_NREAL = 2 * TC_BNC;
 constexpr uint32_t TC_SPIN_LIMIT = 1u << 22;
 
-constexpr int TC_NS = 4;          // MMA stages in the ring
-constexpr int TC_NR = 4;          // raw operand slots (prefetch depth + 1)
+// Two CTAs of short rings per SM instead of one of long rings: a tile of these
+// block shapes has about three K stages, so what bounds the kernel is the
+// latency of each tile's dependent steps (descriptors, gathers, splits,
+// drain), and a second CTA fills it.  A fitted H|psi> at L = 16, D = 256 in split
+// TF32: 8.2 ms of GEMM (one CTA, rings of 4 and 4), 7.9 (two, 2 and 3), 6.8 (two,
+// 2 and 2: the smaller shared memory also leaves more L1 to the gathers);
+// BF16 at L = 24, D = 128: 9.4 -> 7.5 ms; larger blocks, L = 20, D = 640: 45.0 ->
+// 38.6 ms.
+constexpr int TC_CTAS = 2;
+constexpr int TC_NS = 2;          // MMA stages in the ring
+constexpr int TC_NR = 2;          // raw operand slots (prefetch depth + 1)
 constexpr int TC_PROD_WARPS = 8;
 constexpr int TC_PROD = TC_PROD_WARPS * 32;
 constexpr int TC_EPI_WARP0 = 8;
@@ -271,7 +280,7 @@ struct Pend {
 };
 
 template <int MODE>   // 0: TF32, 1: 3xTF32, 2: BF16
-__global__ void __launch_bounds__(TC_THREADS, 1) k_gemm_tc(const GemmTask* __restrict__ tasks,
+__global__ void __launch_bounds__(TC_THREADS, TC_CTAS) k_gemm_tc(const GemmTask* __restrict__ tasks,
                                                          const GemmTerm* __restrict__ terms,
                                                          const TcTile* __restrict__ tiles,
                                                          const GemmSeg* __restrict__ segs,
@@ -754,7 +763,7 @@ void launch_gemm_tc(const GemmTask* d_tasks, const GemmTerm* d_terms, const TcTi
                     const GemmSeg* d_segs, const SegOps* d_segops, int ntiles, int mode, int n_sm,
                     int* d_err, cudaStream_t st) {
   if (ntiles <= 0) return;
-  const int grid = ntiles < n_sm ? ntiles : n_sm;
+  const int grid = ntiles < TC_CTAS * n_sm ? ntiles : TC_CTAS * n_sm;
   const int smem = tc_smem_bytes(mode);
   if (mode == 2) {
     set_smem_limit((const void*)k_gemm_tc<2>, smem);
