@@ -175,9 +175,12 @@ const void* Context::stage_send(size_t bytes) {
     oversize.push_back(b);
     return b->p;
   }
-  TD_CHECK_CUDA(cudaMemcpyAsync(d_ring + ring_off, h_ring + ring_off, bytes,
-                                cudaMemcpyHostToDevice, st));
-  const void* out = d_ring + ring_off;
+  const char* out = h_ring + ring_off;
+  if (bytes > DIRECT_BYTES) {
+    TD_CHECK_CUDA(cudaMemcpyAsync(d_ring + ring_off, h_ring + ring_off, bytes,
+                                  cudaMemcpyHostToDevice, st));
+    out = d_ring + ring_off;
+  }
   ring_off += need;
   return out;
 }
@@ -2799,7 +2802,7 @@ MPSd mps_determinant(Context& c, int L, const uint8_t* occ) {
   for (int i = 0; i < L; ++i) {
     m.sites.push_back(make_site(RowGroups::from_bond(m.bonds[i]), m.bonds[i + 1], c.st, false));
     TD_CHECK_CUDA(cudaMemcpyAsync(m.sites[i].data->p, c.stage(&ones[i], sizeof(double2)),
-                                  sizeof(double2), cudaMemcpyDeviceToDevice, c.st));
+                                  sizeof(double2), cudaMemcpyDefault, c.st));
   }
   m.rcanon = true;   // every site is a single unit entry
   return m;

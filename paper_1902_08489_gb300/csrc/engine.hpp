@@ -89,7 +89,15 @@ struct Context {
   explicit Context(cudaStream_t s, int prec, size_t ring_bytes = (size_t)256 << 20);
   ~Context();
 
-  // copy a host array into device memory valid until the stream passes it
+  // make a host array readable by the kernels of this stream until the stream
+  // passes it.  Lists of up to DIRECT_BYTES stay in the page-locked ring, which
+  // kernels read in place: a copy in front of a kernel costs 5.7 us of stream
+  // time (copy and kernel 9.8 us, kernel alone 4.1), reading a small list over
+  // the CPU link 1 or 2.  Larger lists are copied: their CTAs read more, each
+  // with the link's latency.  Measured with the line at 0 / 4 / 16 / 64 / 256 KB:
+  // two-site Runge-Kutta step at L = 8 151 / 140 / 138 / 137 / 137 ms, <psi|H|phi>
+  // at L = 16, D = 256 7.9 / 7.8 / 7.8 / 7.9 / 8.6 ms.
+  static constexpr size_t DIRECT_BYTES = 16 << 10;
   const void* stage(const void* src, size_t bytes);
   // the same in two steps: room for `bytes` (host memory to fill, before any
   // other staging call), then the copy, which returns the device address

@@ -191,7 +191,7 @@ cplx overlap_noalloc(Context& c, const MPSd& bra, const MPSd& ket) {
   // copy (the ring reuses a segment once the launches that read it are
   // enqueued).
   TD_CHECK_CUDA(cudaMemcpyAsync(Efirst, c.stage(&one, sizeof(one)), sizeof(double2),
-                                cudaMemcpyDeviceToDevice, c.st));
+                                cudaMemcpyDefault, c.st));
   for (const Launch& ln : plan) {
     const char* p = (const char*)c.stage(ln.pack.data(), ln.pack.size());
     launch_gemm((const GemmTask*)p, (const GemmTerm*)(p + ln.o_terms), nullptr, nullptr,
