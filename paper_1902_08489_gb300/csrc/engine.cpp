@@ -561,11 +561,12 @@ struct GemmBatch {
       t.ct = 1;
     }
   }
-  // A launch whose tiles (32 x 32, segments apart) are all of at most
-  // SMALL_MACS complex multiply-adds, and few enough for one wave of that
-  // size, runs on the FP64 pipe (0.43 of them per clock and SM: 9 us; the
-  // sliced kernel takes about as long for any tile).
-  static constexpr long long SMALL_MACS = 8192;
+  // A launch whose blocks (32 x 32, segments apart) are all of at most
+  // SMALL_MACS complex multiply-adds, and few enough for about one wave of
+  // that size, runs on the FP64 pipe (0.43 of them per clock and SM).  Lines
+  // at 4096 / 8192 / 16384 / 24576: five-term sum at L = 12, D = 128 4.45 / 4.41 /
+  // 4.24 / 4.24 ms, FP64 fitted H|psi> at L = 11, D = 117 6.50 / 6.54 / 6.53 / 6.68.
+  static constexpr long long SMALL_MACS = 16384;
   bool small_fp64() const {
     long long total = 0;
     for (const auto& t : tasks) {
@@ -701,7 +702,9 @@ struct GemmBatch {
     // than SMs leaves the rest idle), with at least `min_chunks` K chunks
     // per unit to amortise the partial-slice store and its reduction.
     const int kc = fp64 ? f64_stage_k() : tc_stage_k();
-    const int per_sm = fp64 ? 4 : 3, min_chunks = fp64 ? 2 : 4;
+    // (the small FP64 kernel shares a tile's K among four groups of threads
+    // itself, so it splits later)
+    const int per_sm = fp64 ? 4 : 3, min_chunks = small ? 8 : fp64 ? 2 : 4;
     std::vector<long long>& stages = lists->stages;
     stages.assign(tasks.size(), 0);
     long long total = 0;
