@@ -116,6 +116,8 @@ Context::Context(cudaStream_t s, int prec, size_t ring_bytes) : st(s), precision
   ring_cap = seg_cap * RING_SEGS;
   for (int k = 0; k < RING_SEGS; ++k)
     TD_CHECK_CUDA(cudaEventCreateWithFlags(&seg_ev[k], cudaEventDisableTiming));
+  TD_CHECK_CUDA(cudaEventCreateWithFlags(&copy_ev, cudaEventDisableTiming));
+  TD_CHECK_CUDA(cudaStreamCreateWithFlags(&copy_st, cudaStreamNonBlocking));
   TD_CHECK_CUDA(cudaGetDevice(&device));
   TD_CHECK_CUDA(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, device));
   TD_CHECK_CUDA(cudaMallocHost((void**)&h_ring, ring_cap));
@@ -134,6 +136,9 @@ Context::~Context() {
   rdm.reset();
   status.reset();
   cudaStreamSynchronize(st);
+  if (copy_st) cudaStreamSynchronize(copy_st);
+  if (copy_st) cudaStreamDestroy(copy_st);
+  if (copy_ev) cudaEventDestroy(copy_ev);
   if (h_ring) cudaFreeHost(h_ring);
   if (d_ring) cudaFree(d_ring);
   for (int k = 0; k < RING_SEGS; ++k)
@@ -178,7 +183,9 @@ const void* Context::stage_send(size_t bytes) {
   const char* out = h_ring + ring_off;
   if (bytes > DIRECT_BYTES) {
     TD_CHECK_CUDA(cudaMemcpyAsync(d_ring + ring_off, h_ring + ring_off, bytes,
-                                  cudaMemcpyHostToDevice, st));
+                                  cudaMemcpyHostToDevice, copy_st));
+    TD_CHECK_CUDA(cudaEventRecord(copy_ev, copy_st));
+    TD_CHECK_CUDA(cudaStreamWaitEvent(st, copy_ev, 0));
     out = d_ring + ring_off;
   }
   ring_off += need;
