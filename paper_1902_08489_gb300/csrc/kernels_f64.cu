@@ -13,13 +13,19 @@
 //     (62 fractional bits; an FP64 number within 2^9 of the row's largest
 //     enters unrounded);
 //   * the integer products d_p e_q with p + q = s are added into one FP32
-//     accumulator per s.  |d e| <= 2^16 and at most 64 real K and s + 1 pairs
-//     give at most (s + 1) 2^22, so the sums stay exact (<= 2^24) for s <= 3
-//     and are rounded below 2^-59 of the row-column scale after that;
-//     s = 0 .. 6 is kept, what is dropped is below 2^-60 per product;
+//     accumulator per s = 0 .. 6.  |d e| <= 2^16 and at most 64 real K and s + 1
+//     pairs give at most (s + 1) 2^22, so the sums are exact (<= 2^24) for s <= 3;
+//     from s = 4 on (units of 2^-52 and less of row times column scale) they could
+//     reach 7 2^22 and round to the next even integer, if all digits of all
+//     products were near 256 and of one sign.  Dropped are s >= 7, at most 0.75
+//     2^-60 per real product, and the operands' bits below 2^-62, 0.5 2^-60;
 //   * the seven sums of an output become one 64-bit integer, that one an
 //     FP64 number, and only the sum over K groups and terms is FP64
 //     arithmetic (one addition per group).
+// These errors are relative to the row's largest element times the column's.  An
+// output whose own products are all far below that, as in a state whose bonds
+// are not balanced, is added up on the FP64 pipe instead (OZ_LEAD below), so
+// that the error is that of FP64 sums everywhere.
 // A complex product takes the real 2x2 form: one k16 MMA step holds 8 complex
 // k of op(A) as (re, im) pairs; complex column n of op(B) is stored as the real
 // columns 2n, (br, -bi) pairs, and 2n + 1, (bi, br) pairs.
@@ -30,11 +36,14 @@
 // grain wastes less than tcgen05's 128 rows; the slices are also made where
 // they are used.
 //
-// What bounds it: instruction issue (2 per clock and SM of 4) of the slicing
-// and of the sums' conversion; the tensor pipe is about 10% busy.  Measured
-// on <psi|H|phi> at L = 16, D = 256 (32 launches, 7.2 GFLOP): 4.2 ms, where the
-// FP64 pipe's kernel took 9.7 ms; the error against 64 bits of the adjoint
-// energy gradient at L = 12, D = 128 went from 2.9e-15 to 1.7e-15.
+// What bounds it: latency.  Two CTAs of 8 warps per SM (shared memory) go through
+// load, slice and multiply phases with a barrier after each: 38% of the issue
+// slots and 24% of the warps are busy, the tensor pipe about 10%.  Measured
+// on <psi|H|phi> at L = 16, D = 256 (32 launches, 7.2 GFLOP): 4.4 ms, where the
+// FP64 pipe's kernel took 9.7 ms (4.1 without the FP64 pipe for single outputs,
+// whose results were wrong there); the same with bonds rescaled by 2^+-20, where
+// everything goes to the FP64 pipe: 11.3 ms; the error against 64 bits of the
+// adjoint energy gradient at L = 12, D = 128 is 1.7e-15 (FP64 pipe: 2.9e-15).
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -56,10 +65,17 @@ constexpr int OZ_KC = 32;       // complex K per group
 constexpr int OZ_THREADS = 256;
 constexpr int OZ_WA = OZ_M * OZ_KC, OZ_WB = 2 * OZ_N * OZ_KC;   // half2 words of one slice
 constexpr int OZ_SMEM = OZ_S * (OZ_WA + OZ_WB) * 4;          // A and B slices
+constexpr int OZ_LD = OZ_KC + 1;   // complex FP64 row in shared memory (OzFrag::stage)
+static_assert((OZ_M + OZ_N) * OZ_LD * 16 <= OZ_SMEM, "staged numbers take the slices' place");
 constexpr int OZ_INF = 0x7ff;
 
 __device__ __forceinline__ double2 zmul(double2 a, double2 b) {
   return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+}
+
+__device__ __forceinline__ void zfma(double2& c, double2 a, double2 b) {
+  c.x = fma(a.x, b.x, fma(-a.y, b.y, c.x));
+  c.y = fma(a.x, b.y, fma(a.y, b.x, c.y));
 }
 
 __device__ __forceinline__ void mma_f16(float* c, const uint32_t* a, uint32_t b0, uint32_t b1) {
@@ -92,11 +108,12 @@ __device__ __forceinline__ long long madwide(int a, int b, long long c) {
 // rows that one ldmatrix phase reads over all banks
 __device__ __forceinline__ int oz_word(int row, int k) { return row * OZ_KC + (k ^ ((row & 7) << 2)); }
 
-// exponent field of the larger part
-__device__ __forceinline__ int oz_exp(double2 v) {
-  const int a = (__double2hiint(v.x) >> 20) & OZ_INF, b = (__double2hiint(v.y) >> 20) & OZ_INF;
-  return a > b ? a : b;
+// size of a number as an integer that orders like it (0 only for zero); the
+// upper bits are the exponent field
+__device__ __forceinline__ int oz_key(double x) {
+  return (__double2hiint(x) & 0x7FFFFFFF) | (int)min((unsigned)__double2loint(x), 1u);
 }
+__device__ __forceinline__ int oz_exp(int key) { return max(key >> 20, 1); }
 
 // x 2^(1022 - E) as a 62-bit fraction plus the digit bias: sum_j 256 512^j, so
 // that every 9-bit field holds digit + 256
@@ -157,12 +174,11 @@ struct OzFrag {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     return row_op ? lane : warp + 8 * (j / RB);
   }
-  // loads the group (scaled by sc when `scaled`) and leaves the largest
-  // exponent of each row in rexp (zeroed before); a segmented operand has one
+  // loads the group (scaled by sc when `scaled`); a segmented operand has one
   // block per segment of its rows (sg, so non-null)
   __device__ __forceinline__ void load(const void* base, int ld, const GemmSeg* sg,
                                        const SegOps* so, int op, int row0, int rows, int k0, int nk,
-                                       bool row_op, bool scaled, double2 sc, int* rexp) {
+                                       bool row_op, bool scaled, double2 sc) {
 #pragma unroll
     for (int j = 0; j < N; ++j) {
       const int r = row(j, row_op), kk = k(j, row_op);
@@ -187,33 +203,62 @@ struct OzFrag {
 #pragma unroll
       for (int j = 0; j < N; ++j) v[j] = zmul(sc, v[j]);
     }
+  }
+  // leaves the size (oz_key) of the largest part of each row in key[row], and
+  // those of the largest real and imaginary part of all rows in key[part],
+  // key[part + 1] (all zeroed before)
+  __device__ __forceinline__ void sizes(int rows, bool row_op, int* key, int part) const {
+    int re = 0, im = 0;
     if (row_op) {
 #pragma unroll
       for (int j = 0; j < N; ++j) {
         const int r = row(j, true);
         if (r >= rows) break;   // the same for every lane
-        const int e = __reduce_max_sync(0xffffffffu, oz_exp(v[j]));
-        if ((threadIdx.x & 31) == 0) rexp[r] = e;
+        const int x = oz_key(v[j].x), y = oz_key(v[j].y);
+        re = max(re, x);
+        im = max(im, y);
+        const int e = __reduce_max_sync(0xffffffffu, max(x, y));
+        if ((threadIdx.x & 31) == 0) key[r] = e;
       }
     } else {
 #pragma unroll
       for (int b = 0; b < RB; ++b) {
-        int e = 0;
+        int xb = 0, yb = 0;
 #pragma unroll
-        for (int j = b; j < N; j += RB) e = max(e, oz_exp(v[j]));
-        if (e) atomicMax(&rexp[row(b, false)], e);
+        for (int j = b; j < N; j += RB) {
+          xb = max(xb, oz_key(v[j].x));
+          yb = max(yb, oz_key(v[j].y));
+        }
+        const int e = max(xb, yb);
+        if (e) atomicMax(&key[row(b, false)], e);
+        re = max(re, xb);
+        im = max(im, yb);
       }
+    }
+    re = __reduce_max_sync(0xffffffffu, re);
+    im = __reduce_max_sync(0xffffffffu, im);
+    if ((threadIdx.x & 31) == 0) {
+      atomicMax(&key[part], re);
+      atomicMax(&key[part + 1], im);
     }
   }
   // the slices; rows past the block only reach outputs that are never stored,
   // k is zero-filled to the MMA step
   template <bool IS_B>
   __device__ __forceinline__ void slice(uint32_t* s, int rows, int nk8, bool row_op,
-                                        const int* rexp) const {
+                                        const int* key) const {
 #pragma unroll
     for (int j = 0; j < N; ++j) {
       const int r = row(j, row_op), kk = k(j, row_op);
-      if (r < rows && kk < nk8) oz_store<IS_B>(s, r, kk, v[j], max(rexp[r], 1));
+      if (r < rows && kk < nk8) oz_store<IS_B>(s, r, kk, v[j], oz_exp(key[r]));
+    }
+  }
+  // the numbers themselves, [row][k]
+  __device__ __forceinline__ void stage(double2* s, int rows, bool row_op) const {
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      const int r = row(j, row_op);
+      if (r < rows) s[r * OZ_LD + k(j, row_op)] = v[j];
     }
   }
 };
@@ -250,6 +295,87 @@ __device__ __forceinline__ double oz_value(const float (&acc)[OZ_S][4], int c, i
   return oz_double(t, k - 70 + drop);
 }
 
+// What the slices of a group cannot give as accurately as FP64 arithmetic is
+// added up on the FP64 pipe.  The error of the slices is at most 1.25 2^-60 per
+// real product (truncation of both operands, dropped digit products), in units
+// of the row's largest element times the column's; that of FP64 arithmetic is
+// 2^-53 of the product itself.  So
+//   * sum |a| |b| of an output has to reach 1.25 2^-7 of these units.  It does not
+//     where large elements of A only meet small ones of B.  The sum of the
+//     products of the leading digits' magnitudes, over both parts, is at most
+//     4 times it in units of 2^-16 (a leading digit of 1 may stand for a half,
+//     and the parts count a product up to twice);
+//   * each part's scale over the group has to be within 2^-7 of that of both, unless the
+//     part is zero throughout: the imaginary part of nearly real data.
+// Of the outputs of the performance cases 0 to 0.1% fail the first, fewer the
+// second.  A few outputs of a CTA: the warp for each (oz_direct); more than
+// OZ_FEW threads with such outputs: from the numbers in shared memory, and
+// without slices for the rest of the CTA's work once half of the threads have
+// some.  Always from shared memory: the energy gradient above 4.64 ms, with the
+// line at 16 threads 4.55; all from single lanes and global memory: the rescaled
+// <psi|H|phi> 30 ms in all, now 14.8.
+constexpr int OZ_FEW = 16;
+constexpr float OZ_LEAD = 2560.f;   // 4 x 1.25 x 2^-7 x 2^16
+constexpr int OZ_PART = 7;
+// the parts that fail the second rule (bit 0 real, bit 1 imaginary), from the
+// sizes of the largest real and imaginary part of A and of B
+__device__ __forceinline__ int oz_weak_parts(const int* a, const int* b) {
+  constexpr int none = -8192;
+  const int ax = a[0] ? a[0] >> 20 : none, ay = a[1] ? a[1] >> 20 : none;
+  const int bx = b[0] ? b[0] >> 20 : none, by = b[1] ? b[1] >> 20 : none;
+  const int line = max(ax, ay) + max(bx, by) - OZ_PART;
+  const int re = max(ax + bx, ay + by), im = max(ax + by, ay + bx);
+  return (re >= 0 && re < line ? 1 : 0) | (im >= 0 && im < line ? 2 : 0);
+}
+
+enum : int { OZ_ROW_A = 1, OZ_ROW_B = 2, OZ_CONJ_A = 4, OZ_CONJ_B = 8 };
+
+// element (x, k0) of an operand and the stride of its k
+__device__ __forceinline__ void oz_operand(const void* base, int ld, const GemmSeg* sg, const SegOps* so,
+                                           int x, int k0, bool row_op, const double2*& p, size_t& step) {
+  p = (const double2*)base;
+  if (sg) {
+    const int s = (x >= sg->off[1]) + (x >= sg->off[2]) + (x >= sg->off[3]);
+    p = (const double2*)so->p[s];
+    ld = so->ld[s];
+    x -= sg->off[s];
+  }
+  p += row_op ? (size_t)x * ld + k0 : (size_t)k0 * ld + x;
+  step = row_op ? 1 : ld;
+}
+
+// For each lane of a warp with `weak`: the sum of its output (r, c) over the
+// kn <= 32 complex k of one group from k0 on the FP64 pipe, k per lane (a launch
+// waits for the last, and one lane alone takes 3 us for 32 k).
+__device__ __forceinline__ double2 oz_direct(const GemmTerm& tr, const GemmSeg* sgA, const GemmSeg* sgB,
+                                             const SegOps* so, int mode, double2 sc, bool scaled, int r,
+                                             int c, int k0, int kn, bool weak) {
+  const int lane = threadIdx.x & 31;
+  double2 mine = make_double2(0.0, 0.0);
+  for (unsigned todo = __ballot_sync(0xffffffffu, weak); todo; todo &= todo - 1) {
+    const int o = __ffs((int)todo) - 1;
+    const double2 *a, *b;
+    size_t sa, sb;
+    oz_operand(tr.A, tr.lda, sgA, so, __shfl_sync(0xffffffffu, r, o), k0, mode & OZ_ROW_A, a, sa);
+    oz_operand(tr.B, tr.ldb, sgB, so, __shfl_sync(0xffffffffu, c, o), k0, mode & OZ_ROW_B, b, sb);
+    double2 s = make_double2(0.0, 0.0);
+    if (lane < kn) {
+      double2 x = a[lane * sa], y = b[lane * sb];
+      if (mode & OZ_CONJ_A) x.y = -x.y;
+      if (mode & OZ_CONJ_B) y.y = -y.y;
+      if (scaled) x = zmul(sc, x);
+      s = zmul(x, y);
+    }
+#pragma unroll
+    for (int w = 1; w < 32; w <<= 1) {
+      s.x += __shfl_xor_sync(0xffffffffu, s.x, w);
+      s.y += __shfl_xor_sync(0xffffffffu, s.y, w);
+    }
+    if (lane == o) mine = s;
+  }
+  return mine;
+}
+
 // tiles of one dimension: as few as fit, of equal size rounded up to the
 // subtile's
 __host__ __device__ inline int oz_tiles(int n, int most) { return (n + most - 1) / most; }
@@ -283,10 +409,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 2) k_gemm(const GemmTask* __restri
                                                         const GemmSeg* __restrict__ segs,
                                                         const SegOps* __restrict__ segops,
                                                         const int* __restrict__ tile_task) {
-  extern __shared__ uint32_t oz_sh[];
+  extern __shared__ __align__(16) uint32_t oz_sh[];
   uint32_t* sA = oz_sh;
   uint32_t* sB = oz_sh + OZ_S * OZ_WA;
-  __shared__ int rexpA[2][OZ_M], rexpB[2][32];   // exponents of the rows of A and the columns of B
+  // sizes of the rows of A, the columns of B, then of their parts (OzFrag::load)
+  __shared__ int keyA[2][OZ_M + 2], keyB[2][32 + 2];
   const GemmTask& t = tasks[tile_task[blockIdx.x]];
   const unsigned local = blockIdx.x - t.tile_base, splits = t.splits;
   unsigned split = 0, rest = local;
@@ -327,11 +454,17 @@ __global__ void __launch_bounds__(OZ_THREADS, 2) k_gemm(const GemmTask* __restri
     alpha = make_double2((alpha.x * b.x + alpha.y * b.y) / d, (alpha.y * b.x - alpha.x * b.y) / d);
   }
   const bool unit = alpha.x == 1.0 && alpha.y == 0.0;
-  if (threadIdx.x < OZ_M) rexpA[0][threadIdx.x] = 0;
-  if (threadIdx.x < 32) rexpB[0][threadIdx.x] = 0;
+  if (threadIdx.x < OZ_M + 2) keyA[0][threadIdx.x] = 0;
+  if (threadIdx.x < 32 + 2) keyB[0][threadIdx.x] = 0;
   __syncthreads();
   int bufA = 0, bufB = 0;
+  bool sliced_a = false, plain = false;   // the same in all threads
+  double2* xA = (double2*)oz_sh;
+  double2* xB = xA + OZ_M * OZ_LD;
   const int nsm = (rows + 15) >> 4;
+  const int mode = (rowA ? OZ_ROW_A : 0) | (rowB ? OZ_ROW_B : 0) |
+                   (opA == OP_C || opA == OP_J ? OZ_CONJ_A : 0) |
+                   (opB == OP_C || opB == OP_J ? OZ_CONJ_B : 0);
   // the column tiles of this CTA: one, or (walk > 1: a task of one K group)
   // several that share the slices of A
   for (int w = 0; w < walk; ++w) {
@@ -368,71 +501,129 @@ __global__ void __launch_bounds__(OZ_THREADS, 2) k_gemm(const GemmTask* __restri
         const int s0 = c0 + (int)(gi * (unsigned)(c1 - c0) / ng);
         const int s1 = c0 + (int)((gi + 1) * (unsigned)(c1 - c0) / ng);
         const int k0 = s0 * OZ_STAGE, kn8 = (s1 - s0) * OZ_STAGE, kn = min(K - k0, kn8);
-        const int *ra = rexpA[bufA], *rb = rexpB[bufB];
-        {
-          OzFrag<OZ_N> fb;
-          fb.load(tr.B, tr.ldb, sgB, so, opB, n0, cols, k0, kn, rowB, false, sc, rexpB[bufB]);
-          if (w == 0) {
-            OzFrag<OZ_M> fa;
-            fa.load(tr.A, tr.lda, sgA, so, opA, m0, rows, k0, kn, rowA, scaled, sc, rexpA[bufA]);
-            __syncthreads();
-            fa.slice<false>(sA, rows, kn8, rowA, ra);
-            bufA ^= 1;
-          } else {
-            __syncthreads();
+        unsigned todo = ~0u;      // two bits per output: the parts for the FP64 pipe
+        int nweak = OZ_THREADS;   // threads that have some
+        if (!plain) {
+          const int *ra = keyA[bufA], *rb = keyB[bufB];
+          const bool fresh = w == 0 || !sliced_a;
+          {
+            OzFrag<OZ_N> fb;
+            fb.load(tr.B, tr.ldb, sgB, so, opB, n0, cols, k0, kn, rowB, false, sc);
+            fb.sizes(cols, rowB, keyB[bufB], 32);
+            if (fresh) {
+              OzFrag<OZ_M> fa;
+              fa.load(tr.A, tr.lda, sgA, so, opA, m0, rows, k0, kn, rowA, scaled, sc);
+              fa.sizes(rows, rowA, keyA[bufA], OZ_M);
+              __syncthreads();
+              fa.slice<false>(sA, rows, kn8, rowA, ra);
+              bufA ^= 1;
+            } else {
+              __syncthreads();
+            }
+            fb.slice<true>(sB, cols, kn8, rowB, rb);
+            bufB ^= 1;
           }
-          fb.slice<true>(sB, cols, kn8, rowB, rb);
-          bufB ^= 1;
-        }
-        if (w == 0 && threadIdx.x < OZ_M) rexpA[bufA][threadIdx.x] = 0;
-        if (threadIdx.x < 32) rexpB[bufB][threadIdx.x] = 0;
-        if (w > 0) ra = rexpA[bufA ^ 1];   // the exponents the slices were made with
-        __syncthreads();
+          if (fresh && threadIdx.x < OZ_M + 2) keyA[bufA][threadIdx.x] = 0;
+          if (threadIdx.x < 32 + 2) keyB[bufB][threadIdx.x] = 0;
+          if (!fresh) ra = keyA[bufA ^ 1];   // what the slices were made with
+          sliced_a = true;
+          todo = 0;
+          __syncthreads();
+          const int weak_parts = oz_weak_parts(ra + OZ_M, rb + 32);
 #pragma unroll
-        for (int i = 0; i < OZ_SUB; ++i) {
-          if (warp + 8 * i < nsub) {
-            const int nc = sub_col(i), mr = sub_row(i, nc);
-            float acc[OZ_S][4];
+          for (int i = 0; i < OZ_SUB; ++i) {
+            if (warp + 8 * i < nsub) {
+              const int nc = sub_col(i), mr = sub_row(i, nc);
+              float acc[OZ_S][4];
 #pragma unroll
-            for (int s = 0; s < OZ_S; ++s)
+              for (int s = 0; s < OZ_S; ++s)
 #pragma unroll
-              for (int c = 0; c < 4; ++c) acc[s][c] = 0.f;
-            for (int ks = 0; ks < kn8; ks += OZ_STAGE) {
-              const uint32_t wa = aA + 4 * oz_word(mr + la, ks + ka);
-              const uint32_t wb = aB + 4 * oz_word(2 * nc + lr, ks + kb);
-              uint32_t bf[OZ_S][2];
+                for (int c = 0; c < 4; ++c) acc[s][c] = 0.f;
+              float lead[4] = {0.f, 0.f, 0.f, 0.f};
+              for (int ks = 0; ks < kn8; ks += OZ_STAGE) {
+                const uint32_t wa = aA + 4 * oz_word(mr + la, ks + ka);
+                const uint32_t wb = aB + 4 * oz_word(2 * nc + lr, ks + kb);
+                uint32_t bf[OZ_S][2];
 #pragma unroll
-              for (int p = 0; p < OZ_S; ++p) ldmatrix2(bf[p], wb + p * OZ_WB * 4);
+                for (int p = 0; p < OZ_S; ++p) ldmatrix2(bf[p], wb + p * OZ_WB * 4);
 #pragma unroll
-              for (int p = 0; p < OZ_S; ++p) {
-                uint32_t af[4];
-                ldmatrix4(af, wa + p * OZ_WA * 4);
+                for (int p = 0; p < OZ_S; ++p) {
+                  uint32_t af[4];
+                  ldmatrix4(af, wa + p * OZ_WA * 4);
 #pragma unroll
-                for (int r = 0; r + p < OZ_S; ++r) mma_f16(acc[p + r], af, bf[r][0], bf[r][1]);
+                  for (int r = 0; r + p < OZ_S; ++r) mma_f16(acc[p + r], af, bf[r][0], bf[r][1]);
+                  if (p == 0) {   // the leading digits without their signs
+                    constexpr uint32_t mag = 0x7FFF7FFFu;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) af[j] &= mag;
+                    mma_f16(lead, af, bf[0][0] & mag, bf[0][1] & mag);
+                  }
+                }
+              }
+              // accumulators 0, 1: row g, complex column q; 2, 3: row g + 8
+              const int eb = oz_exp(rb[nc + q]);
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                const int mh = mr + g + 8 * h;
+                const int ea = oz_exp(ra[mh]);
+                const int k = ea + eb - 2 * 1022;
+                double2 v = make_double2(oz_value(acc, 2 * h, k), oz_value(acc, 2 * h + 1, k));
+                // a zero row or column needs nothing
+                const int weak = ra[mh] == 0 || rb[nc + q] == 0          ? 0
+                                 : lead[2 * h] + lead[2 * h + 1] < OZ_LEAD ? 3
+                                                                          : weak_parts;
+                if (weak & 1) v.x = 0.0;
+                if (weak & 2) v.y = 0.0;
+                todo |= (unsigned)weak << (2 * (2 * i + h));
+                // an infinity or NaN in the row or the column
+                if (ea == OZ_INF || eb == OZ_INF) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
+                // the first group needs no addition (out is zero): a real branch,
+                // so that the FP64 pipe is left alone
+                if (!first) {
+                  asm volatile("");
+                  v.x += out[i][h].x;
+                  v.y += out[i][h].y;
+                }
+                out[i][h] = v;
               }
             }
-            // accumulators 0, 1: row g, complex column q; 2, 3: row g + 8
-            const int eb = rb[nc + q];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              const int ea = ra[mr + g + 8 * h];
-              const int k = max(ea, 1) + max(eb, 1) - 2 * 1022;
-              double2 v = make_double2(oz_value(acc, 2 * h, k), oz_value(acc, 2 * h + 1, k));
-              // an infinity or NaN in the row or the column
-              if (ea == OZ_INF || eb == OZ_INF) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
-              // the first group needs no addition (out is zero): a real branch,
-              // so that the FP64 pipe is left alone
-              if (!first) {
-                asm volatile("");
-                v.x += out[i][h].x;
-                v.y += out[i][h].y;
-              }
-              out[i][h] = v;
-            }
           }
+          nweak = __syncthreads_count(todo != 0);
         }
         first = false;
-        __syncthreads();
+        if (nweak == 0) continue;
+        const bool stage = nweak > OZ_FEW;
+        if (stage) {
+          OzFrag<OZ_M> fa;
+          fa.load(tr.A, tr.lda, sgA, so, opA, m0, rows, k0, kn, rowA, scaled, sc);
+          fa.stage(xA, rows, rowA);
+          OzFrag<OZ_N> fb;
+          fb.load(tr.B, tr.ldb, sgB, so, opB, n0, cols, k0, kn, rowB, false, sc);
+          fb.stage(xB, cols, rowB);
+          sliced_a = false;
+          plain = nweak > OZ_THREADS / 2;
+          __syncthreads();
+        }
+#pragma unroll 1
+        for (int o = 0; o < 2 * OZ_SUB; ++o) {
+          const int weak = warp + 8 * (o >> 1) < nsub ? (int)(todo >> (2 * o)) & 3 : 0;
+          if (!__any_sync(0xffffffffu, weak)) continue;
+          const int nc = sub_col(o >> 1), mr = sub_row(o >> 1, nc) + g + 8 * (o & 1);
+          double2 d = make_double2(0.0, 0.0);
+          if (stage) {
+            const double2 *a = xA + mr * OZ_LD, *b = xB + (nc + q) * OZ_LD;
+            for (int x = 0; x < kn; ++x) zfma(d, a[x], b[x]);
+          } else {
+            d = oz_direct(tr, sgA, sgB, so, mode, sc, scaled, m0 + mr, n0 + nc + q, k0, kn, weak);
+          }
+#pragma unroll
+          for (int i = 0; i < 2 * OZ_SUB; ++i)
+            if (o == i) {
+              if (weak & 1) out[i >> 1][i & 1].x += d.x;
+              if (weak & 2) out[i >> 1][i & 1].y += d.y;
+            }
+        }
+        if (stage) __syncthreads();
       }
     }
 #pragma unroll
@@ -469,11 +660,6 @@ __global__ void __launch_bounds__(OZ_THREADS, 2) k_gemm(const GemmTask* __restri
 // a small overlap (L = 8, D = 32) 286 -> 230 us, a five-term sum at L = 12,
 // D = 128 4.70 -> 4.24 ms.
 constexpr int ST = 16, SK = 8, SG = 4, STERMS = 32;
-
-__device__ __forceinline__ void zfma(double2& c, double2 a, double2 b) {
-  c.x = fma(a.x, b.x, fma(-a.y, b.y, c.x));
-  c.y = fma(a.x, b.y, fma(a.y, b.x, c.y));
-}
 
 __global__ void __launch_bounds__(64 * SG) k_gemm_small(const GemmTask* __restrict__ tasks,
                                                         const GemmTerm* __restrict__ terms,
