@@ -1164,6 +1164,8 @@ constexpr int QR_THREADS = 128;
 constexpr int QR_CS = 8;
 constexpr double QR_CLUSTER_WORK = 12000;   // m n^2 from which a matrix gets a cluster
 constexpr int QR_SMEM = 200 * 1024;
+constexpr double QR_SQ_MIN = 0x1p-800, QR_SQ_MAX = 0x1p800;   // largest squared norm used as it is
+constexpr double QR_SHIFT = 0x1p700;
 constexpr int QR_BATCH = 512;         // columns of one reduction
 constexpr int QR_BATCH_GLOBAL = 256;  // the same when the matrix stays in global memory
 
@@ -1250,18 +1252,32 @@ __global__ void __launch_bounds__(QR_THREADS) k_qr(const FactTask* __restrict__ 
   if (rank == 0)
     for (int e = tid; e < n * n; e += QR_THREADS) t.V[e] = make_double2(0.0, 0.0);
   __syncthreads();
-  for (int c0 = 0; c0 < n; c0 += NB) {
-    const int cnt = min(NB, n - c0);
-    products(nullptr, c0, cnt, true);
-    for (int k = tid; k < cnt; k += QR_THREADS) {
-      orig[c0 + k] = est[c0 + k] = total(k).x;
-      again[c0 + k] = 0;
-    }
-  }
-  __syncthreads();
-  // non-negative FP64 numbers order like their bit patterns
   long long big = 0;
-  for (int c = 0; c < n; ++c) big = max(big, __double_as_longlong(orig[c]));
+  double back = 1.0;   // what R is multiplied with in the end
+  for (int pass = 0;; ++pass) {
+    for (int c0 = 0; c0 < n; c0 += NB) {
+      const int cnt = min(NB, n - c0);
+      products(nullptr, c0, cnt, true);
+      for (int k = tid; k < cnt; k += QR_THREADS) {
+        orig[c0 + k] = est[c0 + k] = total(k).x;
+        again[c0 + k] = 0;
+      }
+    }
+    __syncthreads();
+    // non-negative FP64 numbers order like their bit patterns
+    big = 0;
+    for (int c = 0; c < n; ++c) big = max(big, __double_as_longlong(orig[c]));
+    // Squared norms far out are brought in by a power of two, once (the same
+    // decision in every CTA): an accepted pivot is down to 1e-24 of the largest
+    // square, and its reciprocal has to be a number.
+    const bool tiny = big < __double_as_longlong(QR_SQ_MIN);
+    if (pass || (!tiny && big <= __double_as_longlong(QR_SQ_MAX))) break;
+    const double f = tiny ? QR_SHIFT : 1.0 / QR_SHIFT;
+    back = 1.0 / f;
+    for (int c = tid >> 5; c < n; c += QR_THREADS / 32)
+      for (int i = tid & 31; i < ml; i += 32) A[c * lda + i] = cscale(A[c * lda + i], f);
+    __syncthreads();
+  }
 
   int nq = 0;
   for (int j = 0; j < n && nq < kmax; ++j) {
@@ -1359,7 +1375,7 @@ __global__ void __launch_bounds__(QR_THREADS) k_qr(const FactTask* __restrict__ 
   if (rank == 0)
     for (int e = tid; e < n * n; e += QR_THREADS) {
       const int q = e % n;
-      if (q < nq) t.V[e] = cscale(t.V[e], est[q]);
+      if (q < nq) t.V[e] = cscale(cscale(t.V[e], est[q]), back);
     }
   // no CTA may leave while others can still write into its slots
   if (CS > 1) cl.sync();
