@@ -151,7 +151,9 @@ __global__ void __launch_bounds__(256) k_wstage(const WTask* __restrict__ tasks,
 // input channel that one of them uses, with its WS_GROUP values (zero where a
 // channel does not use it): four loads feed 16 multiply-adds, where the rows
 // of the single channels took four loads for four.  Every output sums its
-// inputs in the same order as the CSR row (the added products are zeros).
+// inputs in the same order as the CSR row; the zeros are skipped, so that an
+// infinity in one channel stays out of the others' sums (2.98 ms instead of
+// 2.96 at L = 24, D = 128).
 // Measured against the CSR kernel: the centre-site local operator at L = 16,
 // D = 256 (8 launches) 2.38 -> 1.26 ms, a fitted H|psi> there (47 launches)
 // 3.0 -> 2.0 ms, at L = 24, D = 128 (71) 3.7 -> 3.1 ms.
@@ -195,14 +197,22 @@ __global__ void __launch_bounds__(256) k_wstage_f32(const WTask* __restrict__ ta
 #pragma unroll
         for (int r = 0; r < WS_ROWS; ++r) {
           const float2 x = xp[r * rstride];
-          acc[r][0].x = fmaf(v.x, x.x, acc[r][0].x);
-          acc[r][0].y = fmaf(v.x, x.y, acc[r][0].y);
-          acc[r][1].x = fmaf(v.y, x.x, acc[r][1].x);
-          acc[r][1].y = fmaf(v.y, x.y, acc[r][1].y);
-          acc[r][2].x = fmaf(v.z, x.x, acc[r][2].x);
-          acc[r][2].y = fmaf(v.z, x.y, acc[r][2].y);
-          acc[r][3].x = fmaf(v.w, x.x, acc[r][3].x);
-          acc[r][3].y = fmaf(v.w, x.y, acc[r][3].y);
+          if (v.x != 0.f) {
+            acc[r][0].x = fmaf(v.x, x.x, acc[r][0].x);
+            acc[r][0].y = fmaf(v.x, x.y, acc[r][0].y);
+          }
+          if (v.y != 0.f) {
+            acc[r][1].x = fmaf(v.y, x.x, acc[r][1].x);
+            acc[r][1].y = fmaf(v.y, x.y, acc[r][1].y);
+          }
+          if (v.z != 0.f) {
+            acc[r][2].x = fmaf(v.z, x.x, acc[r][2].x);
+            acc[r][2].y = fmaf(v.z, x.y, acc[r][2].y);
+          }
+          if (v.w != 0.f) {
+            acc[r][3].x = fmaf(v.w, x.x, acc[r][3].x);
+            acc[r][3].y = fmaf(v.w, x.y, acc[r][3].y);
+          }
         }
       }
     }
