@@ -98,8 +98,12 @@ void Inter::build_lookup() const {
     n_g = std::max(n_g, b.g + 1);
   }
   lookup.assign((size_t)n_rg * 5 * n_g, -1);
-  for (int i = 0; i < (int)blocks.size(); ++i)
-    lookup[((size_t)blocks[i].rg * 5 + blocks[i].sig + 1) * n_g + blocks[i].g] = i;
+  for (int i = 0; i < (int)blocks.size(); ++i) {
+    int& at = lookup[((size_t)blocks[i].rg * 5 + blocks[i].sig + 1) * n_g + blocks[i].g];
+    if (at >= 0) throw Error(TDMPS_ERR_SECTOR, "two blocks of one row group, state and channel group");
+    at = i;
+  }
+  n_looked = blocks.size();
 }
 
 // ------------------------------------------------------------------ context

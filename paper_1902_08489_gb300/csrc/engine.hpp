@@ -136,8 +136,7 @@ struct Context {
 // ------------------------------------------------------------------ intermediates
 
 // Block-sparse tensor with blocks rows x W x cols keyed (row group, sigma,
-// channel group, column sector); sigma = -1 for environments.  Blocks are
-// added before the first find().
+// channel group, column sector); sigma = -1 for environments.
 struct Inter {
   struct Blk {
     int rg, sig, g, k;
@@ -150,11 +149,11 @@ struct Inter {
   DevPtr data;
   size_t esz() const { return et ? sizeof(float2) : sizeof(double2); }
   // block (rg, sig, g) with column sector k (charge conservation leaves one k
-  // per (rg, sig, g)), or -1.  The lookup table is made on first use: most
-  // intermediates are only walked.
+  // per (rg, sig, g)), or -1.  The lookup table is made on first use, and again
+  // after blocks were added: most intermediates are only walked.
   int find(int rg, int sig, int g, int k) const {
-    if (lookup.empty() && !blocks.empty()) build_lookup();
-    if (rg >= n_rg || g >= n_g) return -1;
+    if (n_looked != blocks.size()) build_lookup();
+    if (rg < 0 || rg >= n_rg || g < 0 || g >= n_g || sig < -1 || sig > 3) return -1;
     const int id = lookup[((size_t)rg * 5 + sig + 1) * n_g + g];
     return id >= 0 && blocks[id].k == k ? id : -1;
   }
@@ -169,6 +168,7 @@ struct Inter {
  private:
   mutable std::vector<int> lookup;   // [(rg * 5 + sig + 1) * n_g + g]
   mutable int n_rg = 0, n_g = 0;
+  mutable size_t n_looked = 0;   // blocks in the table
   void build_lookup() const;
 };
 
