@@ -109,7 +109,12 @@ void Inter::build_lookup() const {
 // ------------------------------------------------------------------ context
 
 std::unique_ptr<GemmLists> Context::take_gemm_lists() {
-  if (gemm_lists.empty()) return std::make_unique<GemmLists>();
+  if (gemm_lists.empty()) {
+    // room for all that were made: a GemmBatch hands its lists back in its
+    // destructor, which must not allocate
+    gemm_lists.reserve(++n_gemm_lists);
+    return std::make_unique<GemmLists>();
+  }
   std::unique_ptr<GemmLists> l = std::move(gemm_lists.back());
   gemm_lists.pop_back();
   return l;

@@ -82,6 +82,7 @@ struct Context {
   std::vector<cudaEvent_t> event_pool;   // recorded and read back events, reused
   std::vector<char> pack;                // host buffer of task lists larger than a ring segment
   std::vector<std::unique_ptr<GemmLists>> gemm_lists;   // free GEMM lists (engine.cpp)
+  size_t n_gemm_lists = 0;   // made so far: as many as were ever in use at once
   std::unique_ptr<GemmLists> take_gemm_lists();
   // scratch for device status words
   DevPtr status;   // int[16]: [0] SVD convergence, [4..5] Krylov, [8] tensor-core waits
