@@ -391,12 +391,16 @@ def roofline(st, precision, cls=None):
         kern, bound, unit = "k_gemm_tc (tcgen05 grouped complex block GEMM)", "tensor", "TFLOP/s"
         achieved = per_launch(ks["flops"]) / per_launch_s / 1e12
     elif top in ("gemm_fp64", "qr", "svd"):
-        kern = {"gemm_fp64": "k_gemm (FP64 grouped complex block GEMM, integer slices on f16 MMA)",
+        kern = {"gemm_fp64": "k_gemm (FP64 grouped complex block GEMM, integer slices on f16 MMA; "
+                             "with k_gemm_small, the FP64-pipe kernel of its small launches)",
                 "qr": "k_qr (FP64 Gram-Schmidt QR, one classical pass counted)",
                 "svd": "k_svd (FP64 one-sided Jacobi SVD)"}[top]
         peak, src, bound, unit = fp64_peak, src64, "alu", "TFLOP/s"
-        if top == "gemm_fp64":   # 28 products of slices per FP64 product; bound by the slicing
-            peak, src = bf16 / 28.0, tag + " sustained bf16 / 28 slice products"
+        if top == "gemm_fp64":
+            # f16 mma.sync takes 1024 multiply-adds per clock and SM (measured), and an
+            # FP64 product 28 of slices; the kernel is bound by latency below that
+            peak = 152 * 1024 * 2 * peaks.get("sm_max_mhz", 2070.0) * 1e-6 / 28.0
+            src, bound = "f16 mma.sync 1024 FMA/clk/SM at the maximum clock / 28 slice products", "latency"
         achieved = per_launch(ks["flops"]) / per_launch_s / 1e12
     else:
         kern = {"wstage": "k_wstage (sparse MPO-tensor stage)", "other": "k_copy/k_scatter"}[top]

@@ -1,5 +1,6 @@
-// FP64 device kernels of the tdmps library: sparse MPO-tensor application, block gather/scatter, one-sided Jacobi SVD, Gram-Schmidt
-// QR, the truncation rule, and the small Krylov algebra.
+// Device kernels of the tdmps library beside the block GEMMs: sparse MPO-tensor
+// application, block gather/scatter, one-sided Jacobi SVD, Gram-Schmidt QR, the
+// truncation rule, and the small Krylov algebra.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -1088,6 +1089,9 @@ __global__ void __launch_bounds__(SVDC_THREADS) k_svd_cl(const FactTask* __restr
 void launch_svd(const FactTask* d_tasks, int ntasks, int* d_status, cudaStream_t st,
                 size_t max_bytes, const FactTask* h_tasks) {
   if (ntasks <= 0) return;
+  // One kernel per launch: k_svd_small when every matrix of the bond fits it
+  // (SVDS_MAX_N; its comment has both sides), else the cluster kernel if all
+  // fit that one, else one CTA per matrix in global memory.
   {
     size_t need = 0;
     bool all_small = h_tasks != nullptr;
@@ -1103,16 +1107,14 @@ void launch_svd(const FactTask* d_tasks, int ntasks, int* d_status, cudaStream_t
     }
   }
   {
-    // the cluster kernel for square (or tall) matrices with a large one
     const size_t cap_cl = 200 * 1024;
     size_t need = 0;
-    bool large = false, shape_ok = h_tasks != nullptr;
+    bool shape_ok = h_tasks != nullptr;
     for (int i = 0; h_tasks && i < ntasks; ++i) {
       need = std::max(need, svdc_elems(h_tasks[i].m, h_tasks[i].n) * sizeof(double2));
       if (h_tasks[i].m < h_tasks[i].n || h_tasks[i].n > 2048) shape_ok = false;
-      if (h_tasks[i].n >= 24) large = true;
     }
-    if (shape_ok && large && need <= cap_cl) {
+    if (shape_ok && need <= cap_cl) {
       set_smem_limit((const void*)k_svd_cl, (int)cap_cl);
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3((unsigned)(ntasks * SVDC_CS));
@@ -1172,7 +1174,10 @@ void launch_svd(const FactTask* d_tasks, int ntasks, int* d_status, cudaStream_t
 // clusters of 4 CTAs: 3.5 ms.
 constexpr int QR_THREADS = 128;
 constexpr int QR_CS = 8;
-constexpr double QR_CLUSTER_WORK = 12000;   // m n^2 from which a matrix gets a cluster
+// m n^2 from which a matrix gets a cluster.  With the line at 0 / 4000 / 12000 /
+// 30000 / never: QR of a two-site Runge-Kutta step at L = 8, D = 64 17.5 / 15.4 / 15.4 /
+// 14.9 / 14.9 ms, of the fitted H|psi> above 3.38 / 3.31 / 3.38 / 3.57 / 5.39 ms.
+constexpr double QR_CLUSTER_WORK = 12000;
 constexpr int QR_SMEM = 200 * 1024;
 constexpr double QR_SQ_MIN = 0x1p-800, QR_SQ_MAX = 0x1p800;   // largest squared norm used as it is
 constexpr double QR_SHIFT = 0x1p700;
