@@ -400,7 +400,7 @@ def roofline(st, precision, cls=None):
             # f16 mma.sync takes 1024 multiply-adds per clock and SM (measured), and an
             # FP64 product 28 of slices; the kernel is bound by latency below that
             peak = 152 * 1024 * 2 * peaks.get("sm_max_mhz", 2070.0) * 1e-6 / 28.0
-            src, bound = "f16 mma.sync 1024 FMA/clk/SM at the maximum clock / 28 slice products", "latency"
+            src = "f16 mma.sync 1024 FMA/clk/SM at the maximum clock / 28 slice products"
         achieved = per_launch(ks["flops"]) / per_launch_s / 1e12
     else:
         kern = {"wstage": "k_wstage (sparse MPO-tensor stage)", "other": "k_copy/k_scatter"}[top]
