@@ -37,13 +37,14 @@
 // they are used.
 //
 // What bounds it: latency.  Two CTAs of 8 warps per SM (shared memory) go through
-// load, slice and multiply phases with a barrier after each: 38% of the issue
+// load, slice and multiply phases with a barrier after each: 40% of the issue
 // slots and 24% of the warps are busy, the tensor pipe about 10%.  Measured
 // on <psi|H|phi> at L = 16, D = 256 (32 launches, 7.2 GFLOP): 4.4 ms, where the
 // FP64 pipe's kernel took 9.7 ms (4.1 without the FP64 pipe for single outputs,
 // whose results were wrong there); the same with bonds rescaled by 2^+-20, where
 // everything goes to the FP64 pipe: 11.3 ms; the error against 64 bits of the
-// adjoint energy gradient at L = 12, D = 128 is 1.7e-15 (FP64 pipe: 2.9e-15).
+// adjoint energy gradient at L = 12, D = 128 is 0.96e-14, the mean over 24 states
+// (FP64 pipe: 1.13e-14).
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -345,8 +346,9 @@ __device__ __forceinline__ void oz_operand(const void* base, int ld, const GemmS
 }
 
 // For each lane of a warp with `weak`: the sum of its output (r, c) over the
-// kn <= 32 complex k of one group from k0 on the FP64 pipe, k per lane (a launch
-// waits for the last, and one lane alone takes 3 us for 32 k).
+// kn <= 32 complex k of one group from k0 on the FP64 pipe, k per lane: a launch
+// waits for the last of them (59 launches of the energy gradient above: 2.65 ms
+// so, 2.88 with all k on one lane).
 __device__ __forceinline__ double2 oz_direct(const GemmTerm& tr, const GemmSeg* sgA, const GemmSeg* sgB,
                                              const SegOps* so, int mode, double2 sc, bool scaled, int r,
                                              int c, int k0, int kn, bool weak) {
